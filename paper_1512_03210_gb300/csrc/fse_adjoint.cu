@@ -103,8 +103,7 @@ extern "C" fse_status fse_step_adjoint(fse_plan_t P, const void* psi_n, void* g,
       for (int k = 0; k < 4; ++k) x1.dp[4 * v + k] = 2.0 * gv * c[k];
     }
   }
-  const int ncx = P->prec == FSE_F32 ? xpass_ncol<float>(P->nx) : xpass_ncol<double>(P->nx);
-  const int xblocks = (x1.nlines + ncx - 1) / ncx;
+  const int xblocks = x_tiles(P, x1.nlines);
   if (dgamma_n && xblocks > kAdjStride) return fail(P, FSE_ERR_UNSUPPORTED, "adjoint: grid too large");
   if ((st = xpass(P, XP_ADJ1, x1)) != FSE_OK) return st;
   // Kc r, then pass 2: g_u1 = h + 2 q u1

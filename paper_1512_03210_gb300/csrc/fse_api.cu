@@ -211,15 +211,48 @@ void prof_end(fse_plan* P, int kind, cudaEvent_t a) {
   P->recs.push_back({kind, a, b});
 }
 
-fse_status col(fse_plan* P, int kind, int N, int var, const ColArgs& a, const MulArgs& m) {
-  if (!twiddle(P, N)) return fail(P, FSE_ERR_INVALID, "no twiddle table for a column pass length");
+namespace {
+template <typename Real>
+cudaError_t launch_col(int n, int var, const ColArgs& a, const MulArgs& m, const void* tw, cudaStream_t st) {
+  switch (var) {
+    case COL_FWD: return launch_col_var<Real, COL_FWD>(n, a, m, tw, st);
+    case COL_INV: return launch_col_var<Real, COL_INV>(n, a, m, tw, st);
+    case COL_PADF: return launch_col_var<Real, COL_PADF>(n, a, m, tw, st);
+    case COL_CROPI: return launch_col_var<Real, COL_CROPI>(n, a, m, tw, st);
+    case COL_KIN: return launch_col_var<Real, COL_KIN>(n, a, m, tw, st);
+    case COL_KIN2: return launch_col_var<Real, COL_KIN2>(n, a, m, tw, st);
+    case COL_KHAT2: return launch_col_var<Real, COL_KHAT2>(n, a, m, tw, st);
+    default: return launch_col_var<Real, COL_KHAT>(n, a, m, tw, st);
+  }
+}
+}  // namespace
+
+// A column pass along an axis of n points.
+fse_status col(fse_plan* P, int kind, int n, int var, const ColArgs& a, const MulArgs& m) {
+  const void* tw = twiddle(P, var == COL_PADF || var == COL_CROPI || var == COL_KHAT || var == COL_KHAT2 ? 2 * n : n);
+  if (!tw) return fail(P, FSE_ERR_INVALID, "no twiddle table for a column pass length");
   cudaEvent_t ev = prof_begin(P);
-  cudaError_t e = P->prec == FSE_F32
-                      ? launch_colpass<float>(N, var, a, m, twiddle(P, N), P->stream)
-                      : launch_colpass<double>(N, var, a, m, twiddle(P, N), P->stream);
+  cudaError_t e = P->prec == FSE_F32 ? launch_col<float>(n, var, a, m, tw, P->stream)
+                                     : launch_col<double>(n, var, a, m, tw, P->stream);
   prof_end(P, kind, ev);
   return launched(P, e, "column pass");
 }
+
+namespace {
+template <typename Real>
+cudaError_t launch_x(int kind, int nx, const XArgs& a, const void* twn, const void* tw2n, cudaStream_t st) {
+  switch (kind) {
+    case XP_FWD: return launch_xpass<Real, XP_FWD>(nx, a, twn, tw2n, st);
+    case XP_INV: return launch_xpass<Real, XP_INV>(nx, a, twn, tw2n, st);
+    case XP_E: return launch_xpass<Real, XP_E>(nx, a, twn, tw2n, st);
+    case XP_R: return launch_xpass<Real, XP_R>(nx, a, twn, tw2n, st);
+    case XP_ADJ1: return launch_xpass<Real, XP_ADJ1>(nx, a, twn, tw2n, st);
+    case XP_ADJ2: return launch_xpass<Real, XP_ADJ2>(nx, a, twn, tw2n, st);
+    case XP_AL: return launch_xpass<Real, XP_AL>(nx, a, twn, tw2n, st);
+    default: return launch_xpass<Real, XP_A>(nx, a, twn, tw2n, st);
+  }
+}
+}  // namespace
 
 fse_status xpass(fse_plan* P, int kind, const XArgs& a) {
   if (!twiddle(P, P->nx) || !twiddle(P, 2 * P->nx)) return fail(P, FSE_ERR_INVALID, "no twiddle table for the x pass");
@@ -227,28 +260,15 @@ fse_status xpass(fse_plan* P, int kind, const XArgs& a) {
                                FSE_PASS_OTHER, FSE_PASS_OTHER, FSE_PASS_A};
   cudaEvent_t ev = prof_begin(P);
   cudaError_t e = P->prec == FSE_F32
-                      ? launch_xpass<float>(kind, P->nx, a, twiddle(P, P->nx), twiddle(P, 2 * P->nx), P->stream)
-                      : launch_xpass<double>(kind, P->nx, a, twiddle(P, P->nx), twiddle(P, 2 * P->nx), P->stream);
+                      ? launch_x<float>(kind, P->nx, a, twiddle(P, P->nx), twiddle(P, 2 * P->nx), P->stream)
+                      : launch_x<double>(kind, P->nx, a, twiddle(P, P->nx), twiddle(P, 2 * P->nx), P->stream);
   prof_end(P, kinds[kind], ev);
   return launched(P, e, "x pass");
 }
 
-int tiles(fse_plan* P, int N, int ncols) {
-  const int nc = P->prec == FSE_F32 ? colpass_ncol<float>(N) : colpass_ncol<double>(N);
-  return (ncols + nc - 1) / nc;
-}
-
-// Passes over the R2C bins 0..nx of many planes: the last, nearly empty tile
-// of every plane (nx + 1 = k NCOL + 1 bins for the usual sizes) is replaced by
-// tail tiles holding that column of NCOL planes each.
-ColArgs with_tail(fse_plan* P, ColArgs a, int N) {
-  const int nc = P->prec == FSE_F32 ? colpass_ncol<float>(N) : colpass_ncol<double>(N);
-  const int rem = a.ncols % nc;
-  if (a.nplanes > 1 && rem > 0 && 2 * rem <= nc) {
-    a.tiles_per_plane = a.ncols / nc;
-    a.tail = rem;
-  }
-  return a;
+// tiles of an x pass over nlines lines (one reduction partial each)
+int x_tiles(fse_plan* P, int nlines) {
+  return P->prec == FSE_F32 ? xpass_tiles<float>(P->nx, nlines) : xpass_tiles<double>(P->nx, nlines);
 }
 
 XArgs x_args(fse_plan* P, void* psi, void* spec) {
@@ -314,20 +334,18 @@ fse_status kinetic_yz(fse_plan* P, void* psi, double f, double dt) {
   fse_status st;
   if (P->dim == 2) {
     m.lp = 0;
-    m.lr = P->ny;
     m.kin_sr = P->nx / 2 + 1;
     m.scale = 1.0 / ((double)P->nx * P->ny);
-    ColArgs a{psi, 0, P->nx, 1, P->nx, P->ny, P->ny, tiles(P, P->ny, P->nx)};
-    return col(P, FSE_PASS_KIN, P->ny, COL_KIN, a, m);
+    ColArgs a{psi, 0, P->nx, 1, P->nx};
+    return col(P, FSE_PASS_KIN, P->ny, COL_KIN2, a, m);
   }
-  ColArgs ay{psi, (long long)P->nx * P->ny, P->nx, P->nz, P->nx, P->ny, P->ny, tiles(P, P->ny, P->nx)};
+  ColArgs ay{psi, (long long)P->nx * P->ny, P->nx, P->nz, P->nx};
   if ((st = col(P, FSE_PASS_COL, P->ny, COL_FWD, ay, m)) != FSE_OK) return st;
   m.lp = P->ny;
-  m.lr = P->nz;
   m.kin_sp = P->nx / 2 + 1;
   m.kin_sr = (long long)(P->nx / 2 + 1) * (P->ny / 2 + 1);
   m.scale = 1.0 / ((double)P->nx * P->ny * P->nz);
-  ColArgs az{psi, P->nx, (long long)P->nx * P->ny, P->ny, P->nx, P->nz, P->nz, tiles(P, P->nz, P->nx)};
+  ColArgs az{psi, P->nx, (long long)P->nx * P->ny, P->ny, P->nx};
   if ((st = col(P, FSE_PASS_KIN, P->nz, COL_KIN, az, m)) != FSE_OK) return st;
   return col(P, FSE_PASS_COL, P->ny, COL_INV, ay, m);
 }
@@ -360,7 +378,6 @@ fse_status nonlocal_yz(fse_plan* P, void* spec, double ta, double tb, bool integ
   fse_status st;
   if (P->dim == 2) {
     m.lp = 0;
-    m.lr = 2 * P->ny;
     m.dkr = 2 * kPi / (2.0 * (P->p.hi[1] - P->p.lo[1]));
     m.chat_sp = 0;
     m.chat_sr = P->chat_cx;
@@ -376,15 +393,13 @@ fse_status nonlocal_yz(fse_plan* P, void* spec, double ta, double tb, bool integ
       m.q[2] = c * (M[1] - n3 * n3 * d);
       m.q[4] = 2 * c * M[3];
     }
-    ColArgs a{spec, 0, P->sx, 1, P->nx + 1, P->ny, P->ny, tiles(P, 2 * P->ny, P->nx + 1)};
-    return col(P, FSE_PASS_KHAT, 2 * P->ny, COL_KHAT, a, m);
+    ColArgs a{spec, 0, P->sx, 1, P->nx + 1};
+    return col(P, FSE_PASS_KHAT, P->ny, COL_KHAT2, a, m);
   }
-  ColArgs af{spec, (long long)2 * P->ny * P->sx, P->sx, P->nz, P->nx + 1, P->ny, 2 * P->ny,
-             tiles(P, 2 * P->ny, P->nx + 1)};
-  if ((st = col(P, FSE_PASS_PAD, 2 * P->ny, COL_PADF, with_tail(P, af, 2 * P->ny), m)) != FSE_OK) return st;
+  ColArgs af{spec, (long long)2 * P->ny * P->sx, P->sx, P->nz, P->nx + 1};
+  if ((st = col(P, FSE_PASS_PAD, P->ny, COL_PADF, af, m)) != FSE_OK) return st;
   m.lp = 2 * P->ny;
   m.dkp = 2 * kPi / (2.0 * (P->p.hi[1] - P->p.lo[1]));
-  m.lr = 2 * P->nz;
   m.dkr = 2 * kPi / (2.0 * (P->p.hi[2] - P->p.lo[2]));
   m.scale = extra_scale / (8.0 * P->nx * P->ny * P->nz);
   if (m.mode == MUL_COULOMB) {
@@ -399,12 +414,9 @@ fse_status nonlocal_yz(fse_plan* P, void* spec, double ta, double tb, bool integ
     m.q[4] = 2 * c * M[4];
     m.q[5] = 2 * c * M[5];
   }
-  ColArgs ag{spec, P->sx, (long long)2 * P->ny * P->sx, 2 * P->ny, P->nx + 1, P->nz, P->nz,
-             tiles(P, 2 * P->nz, P->nx + 1)};
-  if ((st = col(P, FSE_PASS_KHAT, 2 * P->nz, COL_KHAT, with_tail(P, ag, 2 * P->nz), m)) != FSE_OK) return st;
-  ColArgs ah{spec, (long long)2 * P->ny * P->sx, P->sx, P->nz, P->nx + 1, 2 * P->ny, P->ny,
-             tiles(P, 2 * P->ny, P->nx + 1)};
-  return col(P, FSE_PASS_PAD, 2 * P->ny, COL_CROPI, with_tail(P, ah, 2 * P->ny), m);
+  ColArgs ag{spec, P->sx, (long long)2 * P->ny * P->sx, 2 * P->ny, P->nx + 1};
+  if ((st = col(P, FSE_PASS_KHAT, P->nz, COL_KHAT, ag, m)) != FSE_OK) return st;
+  return col(P, FSE_PASS_PAD, P->ny, COL_CROPI, af, m);
 }
 
 // Host-side checks of one parameter set (shared by fse_plan_create and
@@ -462,8 +474,7 @@ fse_status run_steps(fse_plan* P, void* psi, double t0, int nsteps, const double
   XArgs xe = xa;  // E or XI: also writes the mass partials when renormalising
   if (rn) xe.part = renorm_part(P);
   // tiles of pass E, one mass partial each
-  const int ncx = P->prec == FSE_F32 ? xpass_ncol_x2<float>(P->nx) : xpass_ncol_x2<double>(P->nx);
-  const int xblocks = (xa.nlines + ncx - 1) / ncx;
+  const int xblocks = x_tiles(P, xa.nlines);
   // sub-steps of one step: TS2-GauSum itself, or the fourth-order triple jump
   // w1, w0, w1; the kinetic half steps between sub-steps and between steps merge
   const int nsub = P->p.order == 4 ? 3 : 1;
@@ -591,9 +602,7 @@ fse_status fse_plan_create(const fse_params* prm, void* stream, fse_plan_t* out,
     if (seen) continue;
     P->tw_len.push_back(lens[i]);
     P->tw_off.push_back(off);
-    // (cos, sin) and remainder; float plans also hold their (c, c, s, s)
-    // broadcast copy for the packed column passes
-    off = align256(off + 2 * (size_t)lens[i] * P->csize + (P->prec == FSE_F32 ? 2 * (size_t)lens[i] * 16 : 0));
+    off = align256(off + tw_bytes(lens[i], P->prec == FSE_F64));
   }
   P->off_chat = off;
   const size_t nchat = (size_t)P->chat_cx * (P->ny + 1) * (p.dim == 3 ? P->nz + 1 : 1);

@@ -19,137 +19,10 @@
 #include <vector>
 
 #include "fse.h"
+#include "fse_batch.cuh"
 #include "fse_internal.h"
-#include "fse_launch.cuh"
 
 namespace fse {
-
-struct BatchRun {
-  void* psi;
-  void* spec;
-  const void* kin_half;
-  const void* kin_full;
-  double beta, lam, dt, omega, gx2, gy2;
-};
-
-__device__ __forceinline__ double sin_over_dev(double a, double d) {
-  const double z = a * d;
-  return fabs(z) < 1e-6 ? d * (1.0 - z * z / 6.0) : sin(z) / a;
-}
-
-template <typename Real, int N, int VAR>
-__global__ void __launch_bounds__(ColCfg<Real, N, VAR>::NT, ColCfg<Real, N, VAR>::MINB)
-k_colpass_batch(ColArgs a, MulArgs m, const typename Cplx<Real>::T* __restrict__ tw, const BatchRun* runs,
-                int on_spec, int kin_full, int conj) {
-  const BatchRun r = runs[blockIdx.y];
-  a.data = on_spec ? r.spec : r.psi;
-  if constexpr (VAR == COL_KIN) {
-    m.kin = kin_full ? r.kin_full : r.kin_half;
-    m.conj = conj;
-  } else {
-    m.a0 = r.dt * m.scale;
-    m.f.a0 = (float)m.a0;
-  }
-  colpass_body<Real, N, VAR>(a, m, tw, blockIdx.x);
-}
-
-template <typename Real, int NX, int KIND>
-__global__ void __launch_bounds__(XLaunch<Real, NX, KIND>::NT, XLaunch<Real, NX, KIND>::MINB)
-k_xpass_batch(XArgs a, const typename Cplx<Real>::T* __restrict__ twn, const typename Cplx<Real>::T* __restrict__ tw2n,
-              const BatchRun* runs, const double* t0p, int step) {
-  const BatchRun r = runs[blockIdx.y];
-  a.psi = r.psi;
-  a.spec = a.use_spec ? r.spec : nullptr;
-  if constexpr (KIND == XP_A) {
-    // exact time integral of the rotating harmonic trap over the run's step
-    // (Eq. int_poten); the call's start time t0 is a device scalar, so that a
-    // captured graph of the step sequence serves every call. One thread
-    // evaluates the float64 sines and cosines (GB300's float64 pipe is
-    // narrow) and the block reads the coefficients from shared memory.
-    __shared__ double trap[3];
-    if (threadIdx.x == 0) {
-      const double ta = *t0p + step * r.dt, d = r.dt, mid = 2.0 * ta + d;
-      const double C2 = cos(r.omega * mid) * sin_over_dev(r.omega, d);
-      const double S2 = sin(r.omega * mid) * sin_over_dev(r.omega, d);
-      trap[0] = 0.25 * (r.gx2 * (d + C2) + r.gy2 * (d - C2));
-      trap[1] = 0.25 * (r.gx2 * (d - C2) + r.gy2 * (d + C2));
-      trap[2] = 0.5 * (r.gx2 - r.gy2) * S2;
-    }
-    __syncthreads();
-    a.pa = trap[0];
-    a.pb = trap[1];
-    a.pc = trap[2];
-    a.pe = 0.0;
-    a.beta_dt = r.beta * r.dt;
-    a.lam = r.lam;
-    fill_f32_phase(a);
-  }
-  xpass_any<Real, NX, KIND>(a, twn, tw2n, blockIdx.x);
-}
-
-template <int N, int VAR>
-static cudaError_t colb(const ColArgs& a, const MulArgs& m, const void* tw, const BatchRun* runs, int nr,
-                        int on_spec, int kin_full, int conj, cudaStream_t st) {
-  typedef ColCfg<float, N, VAR> K;
-  const size_t smem = K::smem_bytes(VAR);
-  static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_smem(k_colpass_batch<float, N, VAR>, smem, done);
-  if (e != cudaSuccess) return e;
-  dim3 grid(a.nplanes * a.tiles_per_plane, nr);
-  MulArgs mf = m;
-  fill_f32(mf);
-  k_colpass_batch<float, N, VAR><<<grid, K::NT, smem, st>>>(a, mf, reinterpret_cast<const float2*>(tw), runs, on_spec,
-                                                             kin_full, conj);
-  return cudaGetLastError();
-}
-
-static cudaError_t launch_colb(int N, int mode, const ColArgs& a, const MulArgs& m, const void* tw,
-                               const BatchRun* runs, int nr, int on_spec, int kin_full, int conj, cudaStream_t st) {
-  switch (N) {
-#define FSE_CASE(n)                                                                          \
-  case n:                                                                                    \
-    return mode == 1 ? colb<n, COL_KIN>(a, m, tw, runs, nr, on_spec, kin_full, conj, st)      \
-                     : colb<n, COL_KHAT>(a, m, tw, runs, nr, on_spec, kin_full, conj, st);
-    FSE_COL_SIZES(FSE_CASE)
-#undef FSE_CASE
-    default:
-      return cudaErrorInvalidValue;
-  }
-}
-
-template <int NX, int KIND>
-static cudaError_t xb(const XArgs& a, const void* twn, const void* tw2n, const BatchRun* runs, int nr,
-                      const double* t0, int step, cudaStream_t st) {
-  typedef XLaunch<float, NX, KIND> K;
-  const size_t smem = K::smem_bytes();
-  static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_smem(k_xpass_batch<float, NX, KIND>, smem, done);
-  if (e != cudaSuccess) return e;
-  dim3 grid((a.nlines + K::NCOL - 1) / K::NCOL, nr);
-  XArgs af = a;
-  fill_f32(af);
-  k_xpass_batch<float, NX, KIND><<<grid, K::NT, smem, st>>>(af, reinterpret_cast<const float2*>(twn),
-                                                            reinterpret_cast<const float2*>(tw2n), runs, t0, step);
-  return cudaGetLastError();
-}
-
-static cudaError_t launch_xb(int kind, int nx, const XArgs& a, const void* twn, const void* tw2n,
-                             const BatchRun* runs, int nr, const double* t0, int step, cudaStream_t st) {
-  switch (nx) {
-#define FSE_CASE(n)                                                    \
-  case n:                                                              \
-    switch (kind) {                                                    \
-      case XP_FWD: return xb<n, XP_FWD>(a, twn, tw2n, runs, nr, t0, step, st); \
-      case XP_INV: return xb<n, XP_INV>(a, twn, tw2n, runs, nr, t0, step, st); \
-      case XP_E: return xb<n, XP_E>(a, twn, tw2n, runs, nr, t0, step, st);     \
-      default: return xb<n, XP_A>(a, twn, tw2n, runs, nr, t0, step, st);       \
-    }
-    FSE_X_SIZES(FSE_CASE)
-#undef FSE_CASE
-    default:
-      return cudaErrorInvalidValue;
-  }
-}
 
 const void* twiddle(const fse_plan* P, int L);
 template <typename Real>
@@ -349,20 +222,20 @@ fse_status batch_sequence(fse_batch* B, int nsteps, cudaStream_t st0, long long*
     std::memset(&mk1, 0, sizeof(mk1));
     mk1.mode = MUL_KIN;
     mk1.lx = P->nx;
-    mk1.lr = P->ny;
     mk1.kin_sr = P->nx / 2 + 1;
     mk1.scale = 1.0 / ((double)P->nx * P->ny);
-    ColArgs ck{nullptr, 0, P->nx, 1, P->nx, P->ny, P->ny, tiles(P, P->ny, P->nx)};
+    ColArgs ck{nullptr, 0, P->nx, 1, P->nx};
     MulArgs mk2;
     std::memset(&mk2, 0, sizeof(mk2));
     mk2.mode = MUL_COULOMB;
     mk2.lx = 2 * P->nx;
-    mk2.lr = 2 * P->ny;
     mk2.chat = P->ws_ptr(P->off_chat);
     mk2.chat_cx = P->chat_cx;
     mk2.chat_sr = P->chat_cx;
     mk2.scale = 1.0 / (4.0 * P->nx * P->ny);
-    ColArgs cg{nullptr, 0, P->sx, 1, P->nx + 1, P->ny, P->ny, tiles(P, 2 * P->ny, P->nx + 1)};
+    ColArgs cg{nullptr, 0, P->sx, 1, P->nx + 1};
+    const void* twy = twiddle(P, P->ny);
+    const void* tw2y = twiddle(P, 2 * P->ny);
     auto chk = [&](cudaError_t ee, const char* w) -> fse_status {
       if (ee != cudaSuccess) return bfail(B, FSE_ERR_CUDA, std::string(w) + ": " + cudaGetErrorString(ee));
       ++nl;
@@ -371,18 +244,18 @@ fse_status batch_sequence(fse_batch* B, int nsteps, cudaStream_t st0, long long*
     fse_status s;
     if ((s = chk(launch_xb(XP_FWD, P->nx, xa, twn, tw2n, ddesc, nr, t0, 0, st), "batch x")) != FSE_OK) return s;
     for (int n = 0; n < nsteps; ++n) {
-      if ((s = chk(launch_colb(P->ny, 1, ck, mk1, twiddle(P, P->ny), ddesc, nr, 0, n > 0, 0, st), "batch kinetic")) != FSE_OK)
+      if ((s = chk(launch_colb<COL_KIN2>(P->ny, ck, mk1, twy, ddesc, nr, n > 0, st), "batch kinetic")) != FSE_OK)
         return s;
       if (nl_on) {
         if ((s = chk(launch_xb(XP_E, P->nx, xa, twn, tw2n, ddesc, nr, t0, n, st), "batch density")) != FSE_OK) return s;
-        if ((s = chk(launch_colb(2 * P->ny, 2, cg, mk2, twiddle(P, 2 * P->ny), ddesc, nr, 1, 0, 0, st), "batch kernel")) != FSE_OK)
+        if ((s = chk(launch_colb<COL_KHAT2>(P->ny, cg, mk2, tw2y, ddesc, nr, 0, st), "batch kernel")) != FSE_OK)
           return s;
       } else {
         if ((s = chk(launch_xb(XP_INV, P->nx, xa, twn, tw2n, ddesc, nr, t0, n, st), "batch x")) != FSE_OK) return s;
       }
       if ((s = chk(launch_xb(XP_A, P->nx, xa, twn, tw2n, ddesc, nr, t0, n, st), "batch phase")) != FSE_OK) return s;
     }
-    if ((s = chk(launch_colb(P->ny, 1, ck, mk1, twiddle(P, P->ny), ddesc, nr, 0, 0, 0, st), "batch kinetic")) != FSE_OK)
+    if ((s = chk(launch_colb<COL_KIN2>(P->ny, ck, mk1, twy, ddesc, nr, 0, st), "batch kinetic")) != FSE_OK)
       return s;
     if ((s = chk(launch_xb(XP_INV, P->nx, xa, twn, tw2n, ddesc, nr, t0, nsteps, st), "batch x")) != FSE_OK) return s;
     if (multi) {

@@ -1,0 +1,7 @@
+// fse_col_khat_f64.cu -- column-pass instantiations for double: COL_KHAT, COL_KHAT2.
+#include "fse_launch.cuh"
+
+namespace fse {
+template cudaError_t launch_col_var<double, COL_KHAT>(int, const ColArgs&, const MulArgs&, const void*, cudaStream_t);
+template cudaError_t launch_col_var<double, COL_KHAT2>(int, const ColArgs&, const MulArgs&, const void*, cudaStream_t);
+}  // namespace fse

@@ -2,14 +2,14 @@
 #pragma once
 
 #include <atomic>
+#include <type_traits>
 
 #include "fse_passes.cuh"
 
 namespace fse {
 
-// FFT lengths of the column passes (n and 2n) and of the x passes (n).
-#define FSE_COL_SIZES(X) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512) X(768) X(1024)
-#define FSE_X_SIZES(X) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512)
+// Grid lengths.
+#define FSE_SIZES(X) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512)
 
 // Launch of a step pass with programmatic dependent launch on the previous
 // kernel in the stream (see pass_prologue).
@@ -44,103 +44,97 @@ static cudaError_t allow_smem(F* fn, size_t bytes, std::atomic<unsigned long lon
   return e;
 }
 
-template <typename Real, int N, int VAR>
-static cudaError_t col_launch(const ColArgs& a, const MulArgs& m, const void* tw, cudaStream_t st) {
-  typedef ColCfg<Real, N, VAR> K;
-  typedef typename K::C C;
-  const size_t smem = K::smem_bytes(VAR);
+template <typename Real, int N, int VAR, int NP>
+static cudaError_t col_launch(const ColArgs& a, const MulArgs& m, long long blocks, const void* tw,
+                              cudaStream_t st) {
+  typedef ColCfg<Real, N, VAR, NP> K;
+  typedef typename TwOf<Real>::T C;
   static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_smem(k_colpass<Real, N, VAR>, smem, done);
+  cudaError_t e = allow_smem(k_col<Real, N, VAR, NP>, K::smem(), done);
   if (e != cudaSuccess) return e;
-  const long long blocks = col_blocks(a, K::NCOL);
   if (blocks <= 0) return cudaSuccess;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   MulArgs mf = m;
   fill_f32(mf);
-  return launch_pass(k_colpass<Real, N, VAR>, (unsigned)blocks, K::NT, smem, st, a, mf, reinterpret_cast<const C*>(tw));
+  return launch_pass(k_col<Real, N, VAR, NP>, (unsigned)blocks, K::NT, K::smem(), st, a, mf,
+                     reinterpret_cast<const C*>(tw));
 }
 
-template <typename Real>
-cudaError_t launch_colpass(int N, int var, const ColArgs& a, const MulArgs& m, const void* tw, cudaStream_t st) {
-  switch (N) {
-#define FSE_CASE(n)                                                         \
-  case n:                                                                   \
-    switch (var) {                                                          \
-      case COL_FWD: return col_launch<Real, n, COL_FWD>(a, m, tw, st);      \
-      case COL_INV: return col_launch<Real, n, COL_INV>(a, m, tw, st);      \
-      case COL_PADF: return col_launch<Real, n, COL_PADF>(a, m, tw, st);    \
-      case COL_CROPI: return col_launch<Real, n, COL_CROPI>(a, m, tw, st);  \
-      case COL_KIN: return col_launch<Real, n, COL_KIN>(a, m, tw, st);      \
-      default: return col_launch<Real, n, COL_KHAT>(a, m, tw, st);          \
-    }
-    FSE_COL_SIZES(FSE_CASE)
+// The width of a column pass's tiles: the widest whose tiles give every SM
+// one, else the narrowest: a 128^2 float64 grid has 16 tiles of 8 columns for
+// 152 SMs and 128 of one (step 96 -> 39 us with the x passes split the same
+// way), a 384 x 192 float32 one 24 and 192 (57 -> 26 us). f(width constant, args with the tiling, blocks).
+template <typename Real, int N, int VAR, typename F>
+static cudaError_t col_pick(const ColArgs& a0, int runs, F&& f) {
+  typedef ColShape<Real, N, VAR> W;
+  constexpr int CW = W::CW;
+  constexpr bool TWO = W::TWO;
+  ColArgs a = a0;
+  long long blocks = col_tiles(a, CW * W::wide(), TWO);
+  if (blocks * runs >= kSMs || W::narrow() == W::wide()) return f(std::integral_constant<int, W::wide()>(), a, blocks);
+  if constexpr (W::mid() != W::wide()) {
+    a = a0;
+    blocks = col_tiles(a, CW * W::mid(), TWO);
+    if (blocks * runs >= kSMs) return f(std::integral_constant<int, W::mid()>(), a, blocks);
+  }
+  a = a0;
+  blocks = col_tiles(a, CW * W::narrow(), TWO);
+  return f(std::integral_constant<int, W::narrow()>(), a, blocks);
+}
+
+// One variant of the column pass at every length.
+template <typename Real, int VAR>
+cudaError_t launch_col_var(int n, const ColArgs& a, const MulArgs& m, const void* tw, cudaStream_t st) {
+  switch (n) {
+#define FSE_CASE(n)                                                                                          \
+  case n:                                                                                                    \
+    return col_pick<Real, n, VAR>(a, 1, [&](auto w, const ColArgs& at, long long blocks) {                   \
+      return col_launch<Real, n, VAR, decltype(w)::value>(at, m, blocks, tw, st);                            \
+    });
+    FSE_SIZES(FSE_CASE)
 #undef FSE_CASE
     default:
       return cudaErrorInvalidValue;
   }
 }
 
-template <typename Real> int colpass_ncol(int N) {
-  return col_ncol(N, 2 * (int)sizeof(Real));
-}
-
-template <typename Real, int NX, int KIND>
+template <typename Real, int NX, int LN, int KIND>
 static cudaError_t x_launch(const XArgs& a, const void* twn, const void* tw2n, cudaStream_t st) {
-  typedef XLaunch<Real, NX, KIND> K;
-  typedef typename Cplx<Real>::T C;
-  const size_t smem = K::smem_bytes();
+  typedef XCfg<Real, NX, LN> K;
+  typedef typename TwOf<Real>::T C;
   static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_smem(k_xpass<Real, NX, KIND>, smem, done);
+  cudaError_t e = allow_smem(k_xpass<Real, NX, LN, KIND>, K::smem(), done);
   if (e != cudaSuccess) return e;
-  const int blocks = (a.nlines + K::NCOL - 1) / K::NCOL;
+  const int blocks = (a.nlines + LN - 1) / LN;
   if (blocks <= 0) return cudaSuccess;
   XArgs af = a;
   fill_f32(af);
-  return launch_pass(k_xpass<Real, NX, KIND>, (unsigned)blocks, K::NT, smem, st, af, reinterpret_cast<const C*>(twn),
-                     reinterpret_cast<const C*>(tw2n));
+  return launch_pass(k_xpass<Real, NX, LN, KIND>, (unsigned)blocks, K::NT, K::smem(), st, af,
+                     reinterpret_cast<const C*>(twn), reinterpret_cast<const C*>(tw2n));
 }
 
-template <typename Real>
-cudaError_t launch_xpass(int kind, int nx, const XArgs& a, const void* twn, const void* tw2n,
-                         cudaStream_t st) {
+// One kind of x pass at every length.
+template <typename Real, int KIND>
+cudaError_t launch_xpass(int nx, const XArgs& a, const void* twn, const void* tw2n, cudaStream_t st) {
   switch (nx) {
-#define FSE_CASE(n)                                                   \
-  case n:                                                             \
-    switch (kind) {                                                   \
-      case XP_FWD: return x_launch<Real, n, XP_FWD>(a, twn, tw2n, st); \
-      case XP_INV: return x_launch<Real, n, XP_INV>(a, twn, tw2n, st); \
-      case XP_E: return x_launch<Real, n, XP_E>(a, twn, tw2n, st);     \
-      case XP_R: return x_launch<Real, n, XP_R>(a, twn, tw2n, st);     \
-      case XP_ADJ1: return x_launch<Real, n, XP_ADJ1>(a, twn, tw2n, st); \
-      case XP_ADJ2: return x_launch<Real, n, XP_ADJ2>(a, twn, tw2n, st); \
-      case XP_AL: return x_launch<Real, n, XP_AL>(a, twn, tw2n, st);   \
-      default: return x_launch<Real, n, XP_A>(a, twn, tw2n, st);       \
-    }
-    FSE_X_SIZES(FSE_CASE)
+#define FSE_CASE(n)                                                                              \
+  case n:                                                                                        \
+    return xpass_pick<Real, n>(a.nlines, 1) == XWidths<Real, n>::wide()                          \
+               ? x_launch<Real, n, XWidths<Real, n>::wide(), KIND>(a, twn, tw2n, st)             \
+               : x_launch<Real, n, XWidths<Real, n>::narrow(), KIND>(a, twn, tw2n, st);
+    FSE_SIZES(FSE_CASE)
 #undef FSE_CASE
     default:
       return cudaErrorInvalidValue;
   }
 }
 
-template <typename Real> int xpass_ncol(int nx) {
+template <typename Real> int xpass_tiles(int nx, int nlines) {
   switch (nx) {
 #define FSE_CASE(n) \
   case n:           \
-    return XCfg<Real, n>::NCOL;
-    FSE_X_SIZES(FSE_CASE)
-#undef FSE_CASE
-    default:
-      return 0;
-  }
-}
-
-template <typename Real> int xpass_ncol_x2(int nx) {
-  switch (nx) {
-#define FSE_CASE(n) \
-  case n:           \
-    return XLaunch<Real, n, XP_E>::NCOL;
-    FSE_X_SIZES(FSE_CASE)
+    return (nlines + xpass_pick<Real, n>(nlines, 1) - 1) / xpass_pick<Real, n>(nlines, 1);
+    FSE_SIZES(FSE_CASE)
 #undef FSE_CASE
     default:
       return 0;

@@ -217,8 +217,8 @@ fse_status fft_full(fse_plan* P, void* buf, int dir) {
   std::memset(&m, 0, sizeof(m));
   XArgs xa = x_args(P, buf, nullptr);
   fse_status st;
-  ColArgs ay{buf, (long long)P->nx * P->ny, P->nx, P->nz, P->nx, P->ny, P->ny, tiles(P, P->ny, P->nx)};
-  ColArgs az{buf, P->nx, (long long)P->nx * P->ny, P->ny, P->nx, P->nz, P->nz, tiles(P, P->nz, P->nx)};
+  ColArgs ay{buf, (long long)P->nx * P->ny, P->nx, P->nz, P->nx};
+  ColArgs az{buf, P->nx, (long long)P->nx * P->ny, P->ny, P->nx};
   if (dir < 0) {
     if ((st = xpass(P, XP_FWD, xa)) != FSE_OK) return st;
     if ((st = col(P, FSE_PASS_OTHER, P->ny, COL_FWD, ay, m)) != FSE_OK) return st;
@@ -298,10 +298,9 @@ fse_status observables(fse_plan* P, const void* psi_in, double t, const double* 
     if ((st = nonlocal_yz(P, spec, t, t, false, mdir, 1.0 / ((double)P->nx * P->nx))) != FSE_OK) return st;
     XArgs xr = x_args(P, const_cast<C*>(psi), spec);
     xr.part = part + SL_NON * kPartStride;
-    const int ncx = P->prec == FSE_F32 ? xpass_ncol<float>(P->nx) : xpass_ncol<double>(P->nx);
-    if ((xr.nlines + ncx - 1) / ncx > kPartStride) return fail(P, FSE_ERR_UNSUPPORTED, "observables: grid too large");
+    if (x_tiles(P, xr.nlines) > kPartStride) return fail(P, FSE_ERR_UNSUPPORTED, "observables: grid too large");
     if ((st = xpass(P, XP_R, xr)) != FSE_OK) return st;
-    cnt.n[SL_NON] = (xr.nlines + ncx - 1) / ncx;
+    cnt.n[SL_NON] = x_tiles(P, xr.nlines);
   }
 
   cudaEvent_t ev = prof_begin(P);

@@ -10,14 +10,12 @@
 // full-line value sqrt(pi)/tau exp(-k^2/(4 tau^2)) is used.
 #include <cuda_runtime.h>
 
-#include "fse_fft.cuh"
+#include "fse_vec.cuh"
 
 namespace fse {
 
-// tw[2m] = exp(-2 pi i m / L), m = 0..L-1, from float64 sincospi, and
-// tw[2m+1] the rounded remainder (exact minus tw[2m]). For float tables the
-// pair (c, s) is chosen among the float neighbours of the float64 values as
-// the one with |c + i s| closest to 1.
+// Rounds (c, s) to float: among the float neighbours of the float64 values the
+// pair with |c + i s| closest to 1.
 __device__ __forceinline__ void round_pair(double c, double s, float2* out) {
   const float c0 = (float)c, s0 = (float)s;
   const float cc[2] = {c0, (double)c0 > c ? nextafterf(c0, -2.f) : nextafterf(c0, 2.f)};
@@ -36,22 +34,73 @@ __device__ __forceinline__ void round_pair(double c, double s, float2* out) {
 }
 __device__ __forceinline__ void round_pair(double c, double s, double2* out) { *out = make_double2(c, s); }
 
-// For float tables the broadcast copy for the packed column passes follows at
-// tw + 2L: twb[2m] = (c, c, s, s) of tw[2m] and twb[2m+1] the same of tw[2m+1].
+// (cos, tan) of a float64 twiddle: among the neighbours of the rounded values
+// the pair whose modulus c sqrt(1 + t^2) is closest to 1 (its error would act on
+// the field's norm in every step) and whose angle moves least. A vanishing
+// cosine is replaced by one whose products with the tangent and with any field
+// value are exact to rounding.
+__device__ __forceinline__ double2 tan_pair(double c, double s) {
+  if (fabs(c) < 1e-30) return make_double2(1e-40, s * 1e40);
+  const double t0 = s / c, rest = fma(-t0, c, s) / c;  // tangent and the remainder of its rounding
+  double best = 1e300;
+  double2 r = make_double2(c, t0);
+  for (int i = -1; i <= 1; ++i)
+    for (int j = -1; j <= 1; ++j) {
+      const double cc = i == 0 ? c : nextafter(c, i < 0 ? -2.0 : 2.0);
+      const double tt = j == 0 ? t0 : nextafter(t0, j < 0 ? -1e300 : 1e300);
+      // cc^2 (1 + tt^2) - 1 with the rounding errors of its products and sum
+      const double p = tt * tt, pe = fma(tt, tt, -p);
+      const double q = 1.0 + p, z = q - p, qe = (1.0 - z) + (p - (q - z)) + pe;
+      const double a = cc * cc, ae = fma(cc, cc, -a);
+      const double m = a * q, me = fma(a, q, -m) + a * qe + ae * q;
+      const double cost = fabs(((m - 1.0) + me) * 0.5) + fabs((tt - t0) - rest) / q;
+      if (cost < best) {
+        best = cost;
+        r = make_double2(cc, tt);
+      }
+    }
+  return r;
+}
+
+// The twiddle tables of one transform length (see tw_entries): block y builds
+// the table of plan y / 2 in the radix order y % 2.
 template <typename Real>
-__global__ void k_twiddles(typename Cplx<Real>::T* tw, int L) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= L) return;
+__global__ void k_twiddles(typename TwOf<Real>::T* tw, int L) {
+  constexpr bool F64 = sizeof(Real) == 8;
+  const FftPlan P = (blockIdx.y >> 1) ? fft_plan_slim(L) : fft_plan(L, F64);
+  const bool rev = blockIdx.y & 1;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x, n = tw_entries(L);
+  if (e >= n) return;
+  typename TwOf<Real>::T* t = tw + (long long)blockIdx.y * (F64 ? 1 : 2) * n;
+  // pass p holds R NS entries [r][k]
+  int i = e, ns = P.r[rev ? P.np - 1 : 0], r = 0, k = 0, sub = 1, radix = 1;
+  for (int p = 1; p < P.np; ++p) {
+    const int R = P.r[rev ? P.np - 1 - p : p];
+    if (i < R * ns) {
+      r = i / ns;
+      k = i % ns;
+      sub = R * ns;
+      radix = R;
+      break;
+    }
+    i -= R * ns;
+    ns *= R;
+  }
   double s, c;
-  sincospi(-2.0 * (double)m / (double)L, &s, &c);
-  round_pair(c, s, &tw[2 * m]);
-  // rounded remainder of the exact twiddle (second term of the exact products)
-  tw[2 * m + 1] = mk(Real(c - (double)tw[2 * m].x), Real(s - (double)tw[2 * m].y));
-  if constexpr (sizeof(Real) == 4) {
-    float4* twb = reinterpret_cast<float4*>(tw + 2 * L);
-    const float2 w = tw[2 * m], l = tw[2 * m + 1];
-    twb[2 * m] = make_float4(w.x, w.x, w.y, w.y);
-    twb[2 * m + 1] = make_float4(l.x, l.x, l.y, l.y);
+  sincospi(-2.0 * (double)((long long)k * r % sub) / (double)sub, &s, &c);
+  if constexpr (F64) {
+    if (tw_tan(radix, true)) {
+      t[e] = tan_pair(c, s);
+    } else {
+      t[e] = make_double2(c, s);
+    }
+  } else {
+    float2 w;
+    round_pair(c, s, &w);
+    t[e] = make_float4(w.x, w.x, w.y, w.y);
+    // rounded remainder of the exact twiddle (second term of the exact products)
+    const float lc = (float)(c - (double)w.x), ls = (float)(s - (double)w.y);
+    t[e + n] = make_float4(lc, lc, ls, ls);
   }
 }
 
@@ -168,7 +217,8 @@ __global__ void k_chat(Real* out, const double* w, const double* gx, const doubl
 
 template <typename Real>
 cudaError_t launch_twiddles(void* tw, int L, cudaStream_t st) {
-  k_twiddles<Real><<<(L + 127) / 128, 128, 0, st>>>(reinterpret_cast<typename Cplx<Real>::T*>(tw), L);
+  const dim3 grid((tw_entries(L) + 127) / 128, tw_tables(sizeof(Real) == 8));
+  k_twiddles<Real><<<grid, 128, 0, st>>>(reinterpret_cast<typename TwOf<Real>::T*>(tw), L);
   return cudaGetLastError();
 }
 
