@@ -275,13 +275,12 @@ typedef struct {
   double residual;  /* ||r|| / ||b|| of the last inner solve */
 } fse_gs_info;
 /* Device workspace (bytes, 256-byte aligned) that fse_ground_state needs for
- * its Krylov vectors on this plan: ten complex and three real fields. */
+ * its Krylov vectors on this plan: eight complex and three real fields. */
 fse_status fse_ground_state_workspace(fse_plan_t plan, size_t* bytes);
 /* psi (device, plan layout): initial guess on entry (scaled to unit mass),
- * the last iterate on return. The BiCGStab scalars stay on the device, so
- * the launches of one iteration are captured once per call as a CUDA graph
- * and replayed; the host reads the scalars one iteration behind the GPU (one
- * extra, idempotent iteration may run after convergence). The solve runs on
+ * the last iterate on return. The BiCGStab scalars stay on the device; the
+ * host queues iterations one ahead of the scalars it reads (one extra,
+ * idempotent iteration may run after convergence). The solve runs on
  * a stream the plan creates at the first call, ordered after and before the
  * plan's stream, and the call returns with the plan's stream synchronised. It
  * uses the plan's scratch field and spectrum, and keeps that stream, four

@@ -21,8 +21,8 @@ SOURCES = ["fse_api.cu", "fse_precompute.cu", "fse_observables.cu", "fse_adjoint
            "fse_col_plain_f64.cu", "fse_col_kin_f64.cu", "fse_col_pad_f64.cu", "fse_col_khat_f64.cu",
            "fse_x_e_f32.cu", "fse_x_a_f32.cu", "fse_x_adj_f32.cu", "fse_x_e_f64.cu", "fse_x_a_f64.cu",
            "fse_x_adj_f64.cu", "fse_noalloc.cu", "fse_batch.cu", "fse_batch_col.cu", "fse_batch_x.cu",
-           "fse_ground.cu"]
-HEADERS = ["fse_fft.cuh", "fse_vec.cuh", "fse_col.cuh", "fse_passes.cuh", "fse_launch.cuh", "fse_batch.cuh", "fse_internal.h"]
+           "fse_ground.cu", "fse_gs_f32.cu", "fse_gs_f64.cu"]
+HEADERS = ["fse_fft.cuh", "fse_vec.cuh", "fse_col.cuh", "fse_passes.cuh", "fse_launch.cuh", "fse_gsx.cuh", "fse_batch.cuh", "fse_internal.h"]
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]

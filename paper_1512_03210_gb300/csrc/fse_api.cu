@@ -220,6 +220,9 @@ cudaError_t launch_col(int n, int var, const ColArgs& a, const MulArgs& m, const
     case COL_PADF: return launch_col_var<Real, COL_PADF>(n, a, m, tw, st);
     case COL_CROPI: return launch_col_var<Real, COL_CROPI>(n, a, m, tw, st);
     case COL_KIN: return launch_col_var<Real, COL_KIN>(n, a, m, tw, st);
+    case COL_RMUL: return launch_col_var<Real, COL_RMUL>(n, a, m, tw, st);
+    case COL_DY: return launch_col_var<Real, COL_DY>(n, a, m, tw, st);
+    case COL_LZ: return launch_col_var<Real, COL_LZ>(n, a, m, tw, st);
     case COL_KIN2: return launch_col_var<Real, COL_KIN2>(n, a, m, tw, st);
     case COL_KHAT2: return launch_col_var<Real, COL_KHAT2>(n, a, m, tw, st);
     default: return launch_col_var<Real, COL_KHAT>(n, a, m, tw, st);
@@ -249,6 +252,8 @@ cudaError_t launch_x(int kind, int nx, const XArgs& a, const void* twn, const vo
     case XP_ADJ1: return launch_xpass<Real, XP_ADJ1>(nx, a, twn, tw2n, st);
     case XP_ADJ2: return launch_xpass<Real, XP_ADJ2>(nx, a, twn, tw2n, st);
     case XP_AL: return launch_xpass<Real, XP_AL>(nx, a, twn, tw2n, st);
+    case XP_D: return launch_xpass<Real, XP_D>(nx, a, twn, tw2n, st);
+    case XP_LZ: return launch_xpass<Real, XP_LZ>(nx, a, twn, tw2n, st);
     default: return launch_xpass<Real, XP_A>(nx, a, twn, tw2n, st);
   }
 }
@@ -256,8 +261,8 @@ cudaError_t launch_x(int kind, int nx, const XArgs& a, const void* twn, const vo
 
 fse_status xpass(fse_plan* P, int kind, const XArgs& a) {
   if (!twiddle(P, P->nx) || !twiddle(P, 2 * P->nx)) return fail(P, FSE_ERR_INVALID, "no twiddle table for the x pass");
-  static const int kinds[8] = {FSE_PASS_XFWD, FSE_PASS_XINV, FSE_PASS_E, FSE_PASS_A, FSE_PASS_OTHER,
-                               FSE_PASS_OTHER, FSE_PASS_OTHER, FSE_PASS_A};
+  static const int kinds[10] = {FSE_PASS_XFWD, FSE_PASS_XINV, FSE_PASS_E, FSE_PASS_A, FSE_PASS_OTHER,
+                               FSE_PASS_OTHER, FSE_PASS_OTHER, FSE_PASS_A, FSE_PASS_OTHER, FSE_PASS_OTHER};
   cudaEvent_t ev = prof_begin(P);
   cudaError_t e = P->prec == FSE_F32
                       ? launch_x<float>(kind, P->nx, a, twiddle(P, P->nx), twiddle(P, 2 * P->nx), P->stream)
@@ -370,7 +375,9 @@ fse_status nonlocal_yz(fse_plan* P, void* spec, double ta, double tb, bool integ
     }
   }
   m.lx = 2 * P->nx;
-  m.dkx = 2 * kPi / (2.0 * (P->p.hi[0] - P->p.lo[0]));
+  // spacings of the padded frequencies
+  double dk[3];
+  for (int j = 0; j < 3; ++j) dk[j] = j < P->dim ? kPi / (P->p.hi[j] - P->p.lo[j]) : 0.0;
   m.chat = P->ws_ptr(P->off_chat);
   m.chat_cx = P->chat_cx;
   m.chat_sp = P->chat_cx;
@@ -378,7 +385,6 @@ fse_status nonlocal_yz(fse_plan* P, void* spec, double ta, double tb, bool integ
   fse_status st;
   if (P->dim == 2) {
     m.lp = 0;
-    m.dkr = 2 * kPi / (2.0 * (P->p.hi[1] - P->p.lo[1]));
     m.chat_sp = 0;
     m.chat_sr = P->chat_cx;
     m.scale = extra_scale / (4.0 * P->nx * P->ny);
@@ -389,9 +395,9 @@ fse_status nonlocal_yz(fse_plan* P, void* spec, double ta, double tb, bool integ
       // rotation-invariant n_3 term kept); columns carry k_x, rows k_y
       const double n3 = P->p.dip_n[2], c = 1.5 * m.scale;
       m.a0 = 0.0;
-      m.q[0] = c * (M[0] - n3 * n3 * d);
-      m.q[2] = c * (M[1] - n3 * n3 * d);
-      m.q[4] = 2 * c * M[3];
+      m.q[0] = c * (M[0] - n3 * n3 * d) * dk[0] * dk[0];
+      m.q[2] = c * (M[1] - n3 * n3 * d) * dk[1] * dk[1];
+      m.q[4] = 2 * c * M[3] * dk[0] * dk[1];
     }
     ColArgs a{spec, 0, P->sx, 1, P->nx + 1};
     return col(P, FSE_PASS_KHAT, P->ny, COL_KHAT2, a, m);
@@ -399,20 +405,18 @@ fse_status nonlocal_yz(fse_plan* P, void* spec, double ta, double tb, bool integ
   ColArgs af{spec, (long long)2 * P->ny * P->sx, P->sx, P->nz, P->nx + 1};
   if ((st = col(P, FSE_PASS_PAD, P->ny, COL_PADF, af, m)) != FSE_OK) return st;
   m.lp = 2 * P->ny;
-  m.dkp = 2 * kPi / (2.0 * (P->p.hi[1] - P->p.lo[1]));
-  m.dkr = 2 * kPi / (2.0 * (P->p.hi[2] - P->p.lo[2]));
   m.scale = extra_scale / (8.0 * P->nx * P->ny * P->nz);
   if (m.mode == MUL_COULOMB) {
     m.a0 = d * m.scale;
   } else {
     m.a0 = -d * m.scale;
     const double c = 3.0 * m.scale;
-    m.q[0] = c * M[0];
-    m.q[1] = c * M[1];
-    m.q[2] = c * M[2];
-    m.q[3] = 2 * c * M[3];
-    m.q[4] = 2 * c * M[4];
-    m.q[5] = 2 * c * M[5];
+    m.q[0] = c * M[0] * dk[0] * dk[0];
+    m.q[1] = c * M[1] * dk[1] * dk[1];
+    m.q[2] = c * M[2] * dk[2] * dk[2];
+    m.q[3] = 2 * c * M[3] * dk[0] * dk[1];
+    m.q[4] = 2 * c * M[4] * dk[0] * dk[2];
+    m.q[5] = 2 * c * M[5] * dk[1] * dk[2];
   }
   ColArgs ag{spec, P->sx, (long long)2 * P->ny * P->sx, 2 * P->ny, P->nx + 1};
   if ((st = col(P, FSE_PASS_KHAT, P->nz, COL_KHAT, ag, m)) != FSE_OK) return st;

@@ -24,7 +24,6 @@
 
 namespace fse {
 
-const void* twiddle(const fse_plan* P, int L);
 template <typename Real>
 cudaError_t launch_kin_table(void* half, void* full, int nx, int ny, int nz, double dkx, double dky, double dkz,
                              double s, double m2, double dt, cudaStream_t st);

@@ -7,6 +7,9 @@
 //   COL_CROPI          inverse transform of 2n rows keeping rows [0, n) (density)
 //   COL_KHAT           n rows zero-padded to 2n, fwd . kernel transform . inv, rows [0, n) kept
 //   COL_KIN2 / COL_KHAT2  the same on the y axis of a 2D grid
+//   COL_RMUL           fwd . real spectral factor . inv (ground state)
+//   COL_DY             fwd . i k . inv, out of place (derivative along the axis)
+//   COL_LZ             the same derivative d of psi, not stored: partials of sum x Im(conj(psi) d)
 // The padded variants transform length 2n: their first pass leaves out the
 // zero half of its inputs, their last one computes only the rows that are kept.
 #pragma once
@@ -16,7 +19,7 @@
 namespace fse {
 
 enum { MUL_NONE = 0, MUL_KIN = 1, MUL_COULOMB = 2, MUL_DDI = 3 };
-enum { COL_FWD = 0, COL_INV = 1, COL_PADF = 2, COL_CROPI = 3, COL_KIN = 4, COL_KHAT = 5, COL_KIN2 = 6, COL_KHAT2 = 7 };
+enum { COL_FWD = 0, COL_INV = 1, COL_PADF = 2, COL_CROPI = 3, COL_KIN = 4, COL_KHAT = 5, COL_KIN2 = 6, COL_KHAT2 = 7, COL_RMUL = 8, COL_DY = 9, COL_LZ = 10 };
 
 struct ColArgs {
   void* data;
@@ -27,20 +30,24 @@ struct ColArgs {
   // they cover the first tiles_per_plane * NC columns, and further tiles each
   // take NC consecutive (plane, column) pairs of the `tail` remaining columns
   int tiles_per_plane, tail;
+  void* out;  // COL_DY: the result's buffer
+  double* part;     // COL_LZ: one partial per block
+  double lo, h;     // COL_LZ: coordinate of column i, lo + h i
+  int* blocks_out;  // host: receives the number of blocks (null: not wanted)
 };
 
 struct MulArgs {
   int mode;
   int lx;            // signed-wrap length of the column (x) index; 0 = R2C bin (non-negative)
   int lp;            // signed-wrap length of the plane index (0 = no plane axis)
-  double dkx, dkp, dkr;
+  double dkr;        // COL_DY, COL_LZ: spacing of the axis over its length
   double scale;      // 1/N of the transform
   double a0;         // Coulomb: dt*scale; DDI: -dt*scale
-  double q[6];       // DDI: 3*scale*(Mxx, Myy, Mrr..): see host code (x, plane, row)
+  double q[6];       // DDI: 3*scale*(Mxx, Mpp, Mrr, 2 Mxp, 2 Mxr, 2 Mpr) times the two axes' spacings
   const void* chat;
   long long chat_sp, chat_sr;
   int chat_cx;       // padded length of a C^ row (x bins 0..lx/2, then zeros), a multiple of 4
-  const void* kin;   // kinetic: octant table of exp(-i f theta_k) on |p_j| = 0..n_j/2
+  const void* kin;   // COL_RMUL: octant table of real factors; kinetic: octant table of exp(-i f theta_k) on |p_j| = 0..n_j/2
   long long kin_sp, kin_sr;  // kinetic: octant strides of the plane and row axes
   int conj;          // kinetic: multiply by the conjugate of the table (adjoint)
   // float copies of the scalars above, written by fill_f32 before a launch: a
@@ -48,17 +55,18 @@ struct MulArgs {
   // fields in every thread (double-to-float conversions issue on the narrow
   // FP64 pipe)
   struct {
-    float dkx, dkp, dkr, scale, a0, q[6];
+    float dkr, scale, a0, q[6], qt[6];  // qt: what rounding q to float leaves
   } f;
 };
 
 __host__ __device__ inline void fill_f32(MulArgs& m) {
-  m.f.dkx = (float)m.dkx;
-  m.f.dkp = (float)m.dkp;
   m.f.dkr = (float)m.dkr;
   m.f.scale = (float)m.scale;
   m.f.a0 = (float)m.a0;
-  for (int i = 0; i < 6; ++i) m.f.q[i] = (float)m.q[i];
+  for (int i = 0; i < 6; ++i) {
+    m.f.q[i] = (float)m.q[i];
+    m.f.qt[i] = (float)(m.q[i] - (double)m.f.q[i]);
+  }
 }
 
 // A scalar parameter in the kernel's precision: the double field, or its float copy.
@@ -217,6 +225,15 @@ __device__ __forceinline__ double lane_of(const double (&v)[1]) { return v[0]; }
 __device__ __forceinline__ float2 lane_ld(const float* p) { return *reinterpret_cast<const float2*>(p); }
 __device__ __forceinline__ double lane_ld(const double* p) { return *p; }
 
+// s += Im(conj(u) d) per lane, in float64
+__device__ __forceinline__ void lz_add(const Vec<float2>& u, const Vec<float2>& d, double (&s)[2]) {
+  s[0] += (double)u.re.x * d.im.x - (double)u.im.x * d.re.x;
+  s[1] += (double)u.re.y * d.im.y - (double)u.im.y * d.re.y;
+}
+__device__ __forceinline__ void lz_add(const Vec<double>& u, const Vec<double>& d, double (&s)[1]) {
+  s[0] += u.re * d.im - u.im * d.re;
+}
+
 template <typename Real, int N, int VAR, int NP, bool GATHER, bool PDL>
 __device__ __forceinline__ void col_tile(const ColArgs& a, const MulArgs& m, const typename TwOf<Real>::T* __restrict__ tw,
                                          int bid, int ngat) {
@@ -345,6 +362,57 @@ __device__ __forceinline__ void col_tile(const ColArgs& a, const MulArgs& m, con
     F::template each<RF>(it, [&](int e, int row, int r) {
       if (2 * r < RF) col_st(geo, row * ls, v[e]);
     });
+  } else if constexpr (VAR == COL_RMUL) {
+    F::template each<RF>(it, [&](int e, int row, int) { v[e] = col_ld(geo, row * ls); });
+    F::template run<-1, true, false, false>(v, buf, addr, tw, it);
+    const Real* tab[CW];
+#pragma unroll
+    for (int q = 0; q < CW; ++q)
+      tab[q] = reinterpret_cast<const Real*>(m.kin) +
+               (m.lp ? (long long)abs(wrap_index(geo.plane[q], m.lp)) * m.kin_sp : 0) +
+               abs(wrap_index(min(geo.px[q], m.lx - 1), m.lx));
+    fresh();
+    F::template each<RL>(it, [&](int e, int row, int) {
+      const long long ro = (long long)abs(wrap_index(row, N)) * m.kin_sr;
+      Real t[CW];
+#pragma unroll
+      for (int q = 0; q < CW; ++q) t[q] = __ldg(&tab[q][ro]);
+      const L f = lane_of(t);
+      v[e] = {lmul(f, v[e].re), lmul(f, v[e].im)};
+    });
+    fresh();
+    F::template run<+1, true, true, true>(v, buf, addr, tw, it);
+    fresh();
+    F::template each<RF>(it, [&](int e, int row, int) { col_st(geo, row * ls, v[e]); });
+  } else if constexpr (VAR == COL_DY || VAR == COL_LZ) {
+    F::template each<RF>(it, [&](int e, int row, int) { v[e] = col_ld(geo, row * ls); });
+    F::template run<-1, true, false, false>(v, buf, addr, tw, it);
+    const Real dk = prm<Real>(m.dkr, m.f.dkr);  // includes 1/N
+    F::template each<RL>(it, [&](int e, int row, int) {
+      // the odd factor is zero at the Nyquist index
+      const L k = lbc<L>(2 * row == N ? Real(0) : dk * Real(wrap_index(row, N)));
+      v[e] = {lneg(lmul(k, v[e].im)), lmul(k, v[e].re)};
+    });
+    F::template run<+1, true, true, true>(v, buf, addr, tw, it);
+    fresh();
+    if constexpr (VAR == COL_LZ) {
+      __shared__ double red[32];
+      double s[CW];
+#pragma unroll
+      for (int q = 0; q < CW; ++q) s[q] = 0.0;
+      F::template each<RF>(it, [&](int e, int row, int) { lz_add(col_ld(geo, row * ls), v[e], s); });
+      double t = 0.0;
+#pragma unroll
+      for (int q = 0; q < CW; ++q)
+        if (geo.ok[q]) t += (a.lo + a.h * geo.px[q]) * s[q];
+      t = block_sum(t, red);
+      if (tid == 0) a.part[bid] = t;
+      return;
+    }
+#pragma unroll
+    for (int q = 0; q < CW; ++q) geo.p[q] = reinterpret_cast<C*>(a.out) + (geo.p[q] - reinterpret_cast<C*>(a.data));
+    geo.vec = geo.vec && (reinterpret_cast<uintptr_t>(geo.p[0]) % 16 == 0);
+    F::template each<RF>(it, [&](int e, int row, int) { col_st(geo, row * ls, v[e]); });
   } else if constexpr (K::S::KIN) {
     F::template each<RF>(it, [&](int e, int row, int) { v[e] = col_ld(geo, row * ls); });
     F::template run<-1, true, false, false>(v, buf, addr, tw, it);
@@ -382,28 +450,36 @@ __device__ __forceinline__ void col_tile(const ColArgs& a, const MulArgs& m, con
     addr.sync();
     fresh();
     const bool ddi = m.mode == MUL_DDI;
+    // integer frequencies: the spacings are in the factors q, and a float plan
+    // adds what rounding them left (a factor 6e-8 off would act on every mode
+    // alike, and the dipolar energy is a small difference of the modes' sums)
     Real Aq[CW], Bq[CW];
 #pragma unroll
     for (int q = 0; q < CW; ++q) {
-      const Real kp = m.lp ? prm<Real>(m.dkp, m.f.dkp) * Real(wrap_index(geo.plane[q], m.lp)) : Real(0);
+      const Real kp = m.lp ? Real(wrap_index(geo.plane[q], m.lp)) : Real(0);
       const Real kpo = (m.lp && 2 * geo.plane[q] == m.lp) ? Real(0) : kp;
-      const Real kx = prm<Real>(m.dkx, m.f.dkx) * Real(geo.px[q]);
+      const Real kx = Real(geo.px[q]);
       const Real kxo = (2 * geo.px[q] == m.lx) ? Real(0) : kx;
       Aq[q] = prm<Real>(m.q[0], m.f.q[0]) * kx * kx + prm<Real>(m.q[1], m.f.q[1]) * kp * kp +
               prm<Real>(m.q[3], m.f.q[3]) * kxo * kpo;
       Bq[q] = prm<Real>(m.q[4], m.f.q[4]) * kxo + prm<Real>(m.q[5], m.f.q[5]) * kpo;
+      if constexpr (sizeof(Real) == 4) {
+        Aq[q] += m.f.qt[0] * kx * kx + m.f.qt[1] * kp * kp + m.f.qt[3] * kxo * kpo;
+        Bq[q] += m.f.qt[4] * kxo + m.f.qt[5] * kpo;
+      }
     }
     const L A = lane_of(Aq), B = lane_of(Bq), a0 = lbc<L>(prm<Real>(m.a0, m.f.a0));
     const L q2 = lbc<L>(prm<Real>(m.q[2], m.f.q[2]));
-    const Real dkr = prm<Real>(m.dkr, m.f.dkr);
     F::template each<RL>(it, [&](int e, int row, int r) {
       // signed frequency of the row: row - M from M/2 on
       const bool up = RL % 2 == 0 ? 2 * r >= RL : 2 * row >= M;
       const L cv = lane_ld(&sC[(up ? M - row : row) * NC + addr.g * CW]);
       if (ddi) {
         // an exact sum of small integers; the first is the same for every r of an item
-        const L kr = lbc<L>(dkr * (Real(row - r * (M / RL)) + Real(r * (M / RL) - (up ? M : 0))));
-        const L f = lfma(lfma(kr, lfma(q2, kr, 2 * row == M ? lbc<L>(0.0) : B), A), cv, a0);
+        const L kr = lbc<L>(Real(row - r * (M / RL)) + Real(r * (M / RL) - (up ? M : 0)));
+        L b = 2 * row == M ? lbc<L>(0.0) : B;
+        if constexpr (sizeof(Real) == 4) b = lfma(lbc<L>(m.f.qt[2]), kr, b);
+        const L f = lfma(lfma(kr, lfma(q2, kr, b), A), cv, a0);
         v[e] = {lmul(f, v[e].re), lmul(f, v[e].im)};
       } else {
         const L f = lmul(a0, cv);

@@ -1,7 +1,10 @@
-// fse_col_plain_f64.cu -- column-pass instantiations for double: COL_FWD, COL_INV.
+// fse_col_plain_f64.cu -- column-pass instantiations for double: COL_FWD, COL_INV, COL_RMUL, COL_DY, COL_LZ.
 #include "fse_launch.cuh"
 
 namespace fse {
 template cudaError_t launch_col_var<double, COL_FWD>(int, const ColArgs&, const MulArgs&, const void*, cudaStream_t);
 template cudaError_t launch_col_var<double, COL_INV>(int, const ColArgs&, const MulArgs&, const void*, cudaStream_t);
+template cudaError_t launch_col_var<double, COL_RMUL>(int, const ColArgs&, const MulArgs&, const void*, cudaStream_t);
+template cudaError_t launch_col_var<double, COL_DY>(int, const ColArgs&, const MulArgs&, const void*, cudaStream_t);
+template cudaError_t launch_col_var<double, COL_LZ>(int, const ColArgs&, const MulArgs&, const void*, cudaStream_t);
 }  // namespace fse

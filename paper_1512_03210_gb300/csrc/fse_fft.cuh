@@ -109,4 +109,41 @@ __device__ __forceinline__ double2 unit_mul(double2 v, double c, double s, bool 
   return make_double2(v.x * c - v.y * sc, v.x * sc + v.y * c);
 }
 
+// Deterministic float64 block sum (blockDim.x <= 1024; the last warp may be
+// partly filled); result in thread 0.
+__device__ __forceinline__ double block_sum(double v, double* sh) {
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+  const int lanes = min(32, (int)blockDim.x - 32 * w);
+  const unsigned mask = lanes == 32 ? 0xffffffffu : (1u << lanes) - 1u;
+  for (int o = 16; o > 0; o >>= 1) {
+    const double t = __shfl_down_sync(mask, v, o);
+    if (l + o < lanes) v += t;
+  }
+  __syncthreads();
+  if (l == 0) sh[w] = v;
+  __syncthreads();
+  v = 0.0;
+  if (threadIdx.x == 0)
+    for (int i = 0; i < nw; ++i) v += sh[i];
+  return v;
+}
+
+// Deterministic float64 block sums of K values; sh holds K * blockDim.x
+// doubles. Warp w sums values w, w + nw, ... over the block (a float64 warp
+// instruction holds its scheduler for 64 cycles whatever lanes it has, so the
+// additions are packed into few full warps). out(k, sum) is called by one thread.
+template <int K, typename F> __device__ __forceinline__ void block_sums(const double (&s)[K], double* sh, F&& out) {
+  const int n = blockDim.x, w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = n >> 5;
+#pragma unroll
+  for (int k = 0; k < K; ++k) sh[k * n + threadIdx.x] = s[k];
+  __syncthreads();
+  if (w >= nw) return;  // a partly filled last warp does not take part
+  for (int k = w; k < K; k += nw) {
+    double v = 0.0;
+    for (int i = l; i < n; i += 32) v += sh[k * n + i];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (l == 0) out(k, v);
+  }
+}
+
 }  // namespace fse

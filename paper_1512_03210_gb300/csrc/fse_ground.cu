@@ -17,17 +17,16 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
-#include <complex>
 #include <cstring>
 
 #include "fse.h"
 #include "fse_internal.h"
-#include "fse_passes.cuh"
+#include "fse_gsx.cuh"
 
 namespace fse {
 namespace {
 
-constexpr int kGsBlocks = 1024;  // reduction partials per value
+constexpr int kGsBlocks = 1024;  // blocks of the elementwise kernels, at most
 
 struct GsGrid {
   int nx, ny, nz;
@@ -41,16 +40,15 @@ __device__ __forceinline__ void gs_index(long long i, const GsGrid& g, int& ix, 
   iz = (int)(r / g.ny);
 }
 
-// P_Delta / N on the spectrum: 1 / (N (1/dt + (|k|^2 + m^2)^s / 2)), k signed (Nyquist -n/2)
+// P_Delta / N on the octant |p_j| = 0..n_j/2 of the spectrum: 1 / (N (1/dt + (|k|^2 + m^2)^s / 2))
 template <typename Real>
 __global__ void k_gs_precond_table(Real* pk, GsGrid g, double inv_dt, double s, double m2, double inv_n) {
-  const long long N = (long long)g.nx * g.ny * g.nz;
+  const int hx = g.nx / 2 + 1, hy = g.ny / 2 + 1, hz = g.nz > 1 ? g.nz / 2 + 1 : 1;
+  const long long N = (long long)hx * hy * hz;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    int ix, iy, iz;
-    gs_index(i, g, ix, iy, iz);
-    const int px = ix < g.nx / 2 ? ix : ix - g.nx, py = iy < g.ny / 2 ? iy : iy - g.ny;
-    const int pz = g.nz > 1 ? (iz < g.nz / 2 ? iz : iz - g.nz) : 0;
-    const double kx = g.dk[0] * px, ky = g.dk[1] * py, kz = g.dk[2] * pz;
+    const int ix = (int)(i % hx);
+    const long long r = i / hx;
+    const double kx = g.dk[0] * ix, ky = g.dk[1] * (int)(r % hy), kz = g.dk[2] * (int)(r / hy);
     const double k2 = kx * kx + ky * ky + kz * kz + m2;
     pk[i] = Real(inv_n / (inv_dt + 0.5 * (k2 > 0.0 ? pow(k2, s) : 0.0)));
   }
@@ -78,125 +76,44 @@ __global__ void k_gs_potential(const typename Cplx<Real>::T* __restrict__ phi, c
   }
 }
 
-// d = i k_axis sp / N, the odd factor zero at the Nyquist index
+// Partials of sum |a|^2 (float64), part[block]
 template <typename Real>
-__global__ void k_gs_ik(const typename Cplx<Real>::T* __restrict__ sp, typename Cplx<Real>::T* __restrict__ d,
-                        GsGrid g, int axis, double inv_n) {
-  const long long N = (long long)g.nx * g.ny * g.nz;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    int ix, iy, iz;
-    gs_index(i, g, ix, iy, iz);
-    const int idx = axis == 0 ? ix : iy, n = axis == 0 ? g.nx : g.ny;
-    const Real k = (2 * idx == n) ? Real(0) : Real(g.dk[axis] * inv_n) * Real(wrap_index(idx, n));
-    const typename Cplx<Real>::T u = sp[i];
-    d[i] = mk(-k * u.y, k * u.x);
-  }
-}
-
-// out = A_TF u = W u - Omega L_z u = W u + i Omega (x d_y u - y d_x u)
-template <typename Real>
-__global__ void k_gs_atf(const typename Cplx<Real>::T* __restrict__ u, const typename Cplx<Real>::T* __restrict__ dx,
-                         const typename Cplx<Real>::T* __restrict__ dy, const Real* __restrict__ W,
-                         typename Cplx<Real>::T* __restrict__ out, GsGrid g, double omega) {
-  const long long N = (long long)g.nx * g.ny * g.nz;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const typename Cplx<Real>::T a = u[i];
-    const Real w = W[i];
-    Real re = w * a.x, im = w * a.y;
-    if (omega != 0.0) {
-      int ix, iy, iz;
-      gs_index(i, g, ix, iy, iz);
-      const Real x = Real(g.lo[0] + g.h[0] * ix), y = Real(g.lo[1] + g.h[1] * iy);
-      const typename Cplx<Real>::T bx = dx[i], by = dy[i];
-      const Real lr = x * by.x - y * bx.x, li = x * by.y - y * bx.y;  // x d_y u - y d_x u
-      re -= Real(omega) * li;                                          // i Omega (lr + i li)
-      im += Real(omega) * lr;
-    }
-    out[i] = mk(re, im);
-  }
-}
-
-template <typename Real>
-__global__ void k_gs_scale_real(typename Cplx<Real>::T* __restrict__ d, const Real* __restrict__ pk, long long N) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const typename Cplx<Real>::T u = d[i];
-    const Real f = pk[i];
-    d[i] = mk(f * u.x, f * u.y);
-  }
-}
-
-// out = ca A + cb B + cc Cc (complex coefficients; a null operand counts as zero)
-template <typename Real>
-__global__ void k_gs_lincomb(typename Cplx<Real>::T* out, const typename Cplx<Real>::T* A, double2 ca,
-                             const typename Cplx<Real>::T* B, double2 cb, const typename Cplx<Real>::T* Cc, double2 cc,
-                             long long N) {
-  typedef typename Cplx<Real>::T C;
-  const C a = mk(Real(ca.x), Real(ca.y)), b = mk(Real(cb.x), Real(cb.y)), c = mk(Real(cc.x), Real(cc.y));
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    C r = mk(Real(0), Real(0));
-    if (A) r = cadd(r, cmul(A[i], a));
-    if (B) r = cadd(r, cmul(B[i], b));
-    if (Cc) r = cadd(r, cmul(Cc[i], c));
-    out[i] = r;
-  }
-}
-
-// block partials of sum conj(a1) b1 and sum conj(a2) b2 (float64): part[v * kGsBlocks + block], v = 0..3
-template <typename Real>
-__global__ void __launch_bounds__(256) k_gs_dot2(const typename Cplx<Real>::T* a1, const typename Cplx<Real>::T* b1,
-                                                 const typename Cplx<Real>::T* a2, const typename Cplx<Real>::T* b2,
-                                                 long long N, double* part) {
+__global__ void __launch_bounds__(256) k_gs_norm(const typename Cplx<Real>::T* a, long long N, double* part) {
   __shared__ double red[32];
-  double acc[4] = {0, 0, 0, 0};
+  double acc = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const typename Cplx<Real>::T x1 = a1[i], y1 = b1[i], x2 = a2[i], y2 = b2[i];
-    acc[0] += (double)x1.x * y1.x + (double)x1.y * y1.y;
-    acc[1] += (double)x1.x * y1.y - (double)x1.y * y1.x;
-    acc[2] += (double)x2.x * y2.x + (double)x2.y * y2.y;
-    acc[3] += (double)x2.x * y2.y - (double)x2.y * y2.x;
+    const typename Cplx<Real>::T x = a[i];
+    acc += (double)x.x * x.x + (double)x.y * x.y;
   }
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const double t = block_sum(acc[v], red);
-    if (threadIdx.x == 0) part[v * kGsBlocks + blockIdx.x] = t;
-  }
+  acc = block_sum(acc, red);
+  if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
-// block partials of max |a - b|
+// x <- x / ||x|| with ||x||^2 = hd * norm[0], and (old non-null) partials of max |x - old|
 template <typename Real>
-__global__ void __launch_bounds__(256) k_gs_maxdiff(const typename Cplx<Real>::T* a, const typename Cplx<Real>::T* b,
-                                                    long long N, double* part) {
+__global__ void __launch_bounds__(256) k_gs_normalise(typename Cplx<Real>::T* x, const typename Cplx<Real>::T* old,
+                                                      const double* norm, double hd, long long N, double* part) {
   __shared__ double red[256];
+  const Real f = Real(1.0 / sqrt(hd * norm[0]));
   double m = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const double dx = (double)a[i].x - b[i].x, dy = (double)a[i].y - b[i].y;
-    m = fmax(m, sqrt(dx * dx + dy * dy));
+    typename Cplx<Real>::T u = x[i];
+    u = mk(u.x * f, u.y * f);
+    x[i] = u;
+    if (old) {
+      const double dx = (double)u.x - old[i].x, dy = (double)u.y - old[i].y;
+      m = fmax(m, dx * dx + dy * dy);
+      if (!(dx * dx + dy * dy >= 0.0)) m = __longlong_as_double(0x7ff0000000000000LL);  // NaN shows as infinity
+    }
   }
+  if (!old) return;
   red[threadIdx.x] = m;
   __syncthreads();
   for (int o = blockDim.x / 2; o > 0; o >>= 1) {
     if ((int)threadIdx.x < o) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + o]);
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
-}
-
-// out[v] = sum (max = 1: max) over the count partials of value v (one block per value)
-__global__ void __launch_bounds__(256) k_gs_final(const double* part, int count, int max, double* out) {
-  __shared__ double red[256];
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < count; i += blockDim.x) {
-    const double v = part[blockIdx.x * kGsBlocks + i];
-    acc = max ? fmax(acc, v) : acc + v;
-  }
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o)
-      red[threadIdx.x] = max ? fmax(red[threadIdx.x], red[threadIdx.x + o]) : red[threadIdx.x] + red[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[blockIdx.x] = red[0];
+  if (threadIdx.x == 0) part[blockIdx.x] = sqrt(red[0]);
 }
 
 // ---------------------------------------------------------------------------
@@ -204,32 +121,25 @@ __global__ void __launch_bounds__(256) k_gs_final(const double* part, int count,
 //   rho (complex, sc[0..1]), rho_prev (sc[2..3]), alpha (sc[4..5]),
 //   omega (sc[6..7]), beta (sc[8..9]), ||b|| (sc[10]), ||r|| / ||b|| (sc[11]),
 //   done (sc[12]: converged or broken down), iterations (sc[13]), tol (sc[14]).
-// One-thread kernels update it from the inner products in out[] (written by
-// k_gs_final), and the vector updates read their coefficients from it, so an
-// inner iteration needs no host round trip. Once done is set, every update
-// leaves its output untouched.
+// One block sums the partials of an inner product in a fixed order and its
+// first thread updates the state; the vector updates read their coefficients
+// from it, so an inner iteration needs no host round trip. Once done is set,
+// every update leaves its output untouched.
 // ---------------------------------------------------------------------------
-enum { SC_RHO = 0, SC_RHOP = 2, SC_ALPHA = 4, SC_OM = 6, SC_BETA = 8, SC_BN = 10, SC_RES = 11, SC_DONE = 12,
-       SC_IT = 13, SC_TOL = 14, SC_SIZE = 16 };
-
 __device__ __forceinline__ double2 zdiv(double2 a, double2 b) {
   const double d = b.x * b.x + b.y * b.y;
   return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
 }
-__device__ __forceinline__ double2 zmul(double2 a, double2 b) {
-  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ double2 ld2(const double* p) { return make_double2(p[0], p[1]); }
 __device__ __forceinline__ void st2(double* p, double2 v) {
   p[0] = v.x;
   p[1] = v.y;
 }
 
-// after <s, s>, <r, r> (s = b, r = b - M x, rh = r): the start of an inner solve
-__global__ void k_gs_sc_init(double* sc, const double* out, double tol) {
+// after <b, b>, <r, r> (r = b - M x, rh = r): the start of an inner solve
+__device__ __forceinline__ void gs_sc_init(double* sc, const double* out, double tol) {
   const double bn = sqrt(out[0]);
   const double res = bn > 0.0 ? sqrt(out[2]) / bn : 0.0;
-  st2(sc + SC_RHO, make_double2(out[2], out[3]));
+  st2(sc + SC_RHO, make_double2(out[2], 0.0));
   st2(sc + SC_RHOP, make_double2(1.0, 0.0));
   st2(sc + SC_ALPHA, make_double2(1.0, 0.0));
   st2(sc + SC_OM, make_double2(1.0, 0.0));
@@ -238,31 +148,31 @@ __global__ void k_gs_sc_init(double* sc, const double* out, double tol) {
   sc[SC_RES] = res;
   sc[SC_TOL] = tol;
   sc[SC_IT] = 0.0;
-  sc[SC_DONE] = (!(res > tol) || (out[2] == 0.0 && out[3] == 0.0)) ? 1.0 : 0.0;
+  sc[SC_DONE] = (!(res > tol) || out[2] == 0.0) ? 1.0 : 0.0;
 }
 
 // after <rh, v>: alpha = rho / <rh, v> (breakdown when it vanishes)
-__global__ void k_gs_sc_alpha(double* sc, const double* out) {
+__device__ __forceinline__ void gs_sc_alpha(double* sc, const double* out) {
   if (sc[SC_DONE] != 0.0) return;
   const double2 rv = make_double2(out[0], out[1]);
   if (rv.x == 0.0 && rv.y == 0.0) {
     sc[SC_DONE] = 1.0;
     return;
   }
-  st2(sc + SC_ALPHA, zdiv(ld2(sc + SC_RHO), rv));
+  st2(sc + SC_ALPHA, zdiv(gs_ld2(sc + SC_RHO), rv));
 }
 
 // after <t, s>, <t, t>: omega = <t, s> / <t, t> (0 if <t, t> = 0)
-__global__ void k_gs_sc_omega(double* sc, const double* out) {
+__device__ __forceinline__ void gs_sc_omega(double* sc, const double* out) {
   if (sc[SC_DONE] != 0.0) return;
   st2(sc + SC_OM, out[2] > 0.0 ? make_double2(out[0] / out[2], out[1] / out[2]) : make_double2(0.0, 0.0));
 }
 
 // after <rh, r>, <r, r>: the end of an iteration
-__global__ void k_gs_sc_rho(double* sc, const double* out) {
+__device__ __forceinline__ void gs_sc_rho(double* sc, const double* out) {
   if (sc[SC_DONE] != 0.0) return;
-  const double2 rho_prev = ld2(sc + SC_RHO), rho = make_double2(out[0], out[1]);
-  const double2 alpha = ld2(sc + SC_ALPHA), om = ld2(sc + SC_OM);
+  const double2 rho_prev = gs_ld2(sc + SC_RHO), rho = make_double2(out[0], out[1]);
+  const double2 alpha = gs_ld2(sc + SC_ALPHA), om = gs_ld2(sc + SC_OM);
   st2(sc + SC_RHOP, rho_prev);
   st2(sc + SC_RHO, rho);
   const double res = sqrt(out[2]) / sc[SC_BN];
@@ -274,41 +184,67 @@ __global__ void k_gs_sc_rho(double* sc, const double* out) {
     return;
   }
   // beta of the next iteration: (rho / rho_prev) (alpha / omega)
-  st2(sc + SC_BETA, zmul(zdiv(rho, rho_prev), zdiv(alpha, om)));
+  st2(sc + SC_BETA, gs_mul(zdiv(rho, rho_prev), zdiv(alpha, om)));
 }
 
-enum { GS_P = 0, GS_S = 1, GS_X = 2, GS_R = 3 };
-// The BiCGStab vector updates with coefficients from sc (nothing when done):
-//   GS_P: o = A + beta (o - omega Cc)   (o = A on the first iteration)
-//   GS_S: o = A - alpha Cc               GS_X: o = o + alpha A + omega Cc
-//   GS_R: o = A - omega Cc
-template <typename Real, int MODE>
-__global__ void k_gs_update(typename Cplx<Real>::T* o, const typename Cplx<Real>::T* A,
-                            const typename Cplx<Real>::T* Cc, const double* sc, long long N) {
+enum { FIN_SUM = 0, FIN_MAX = 1, FIN_INIT = 2, FIN_ALPHA = 3, FIN_OMEGA = 4, FIN_RHO = 5 };
+// out[v] = sum (FIN_MAX: max) of the count partials of value v, v < nv <= 4 (64
+// threads each, fixed order), then the scalar update that waits for them
+template <int MODE>
+__global__ void __launch_bounds__(256) k_gs_fin(const double* part, int stride, int count, int nv, double* out, double* sc,
+                                                double tol) {
+  pass_prologue();
+  __shared__ double red[256];
+  const int v = threadIdx.x >> 6, t = threadIdx.x & 63;
+  double acc = 0.0;
+  if (v < nv)
+    for (int i = t; i < count; i += 64) {
+      const double x = part[(long long)v * stride + i];
+      acc = MODE == FIN_MAX ? fmax(acc, x) : acc + x;
+    }
+  red[threadIdx.x] = acc;
+  __syncthreads();
+  for (int o = 32; o > 0; o >>= 1) {
+    if (t < o) red[threadIdx.x] = MODE == FIN_MAX ? fmax(acc, red[threadIdx.x + o]) : acc + red[threadIdx.x + o];
+    __syncthreads();
+    acc = red[threadIdx.x];
+  }
+  if (t == 0 && v < nv) out[v] = acc;
+  if (threadIdx.x != 0) return;
+  const double o4[4] = {red[0], red[64], red[128], red[192]};
+  if (MODE == FIN_INIT) gs_sc_init(sc, o4, tol);
+  if (MODE == FIN_ALPHA) gs_sc_alpha(sc, o4);
+  if (MODE == FIN_OMEGA) gs_sc_omega(sc, o4);
+  if (MODE == FIN_RHO) gs_sc_rho(sc, o4);
+}
+
+// The end of an iteration: x += alpha p + omega s, r = s - omega t (nothing
+// when done), and the partials of <rh, r>, <r, r>.
+template <typename Real>
+__global__ void __launch_bounds__(256) k_gs_update(typename Cplx<Real>::T* x, typename Cplx<Real>::T* r,
+                                                   const typename Cplx<Real>::T* p, const typename Cplx<Real>::T* s,
+                                                   const typename Cplx<Real>::T* t, const typename Cplx<Real>::T* rh,
+                                                   const double* sc, long long N, double* part, int stride) {
   typedef typename Cplx<Real>::T C;
-  if (sc[SC_DONE] != 0.0) return;
-  const double2 al = ld2(sc + SC_ALPHA), om = ld2(sc + SC_OM), be = ld2(sc + SC_BETA);
-  const bool first = sc[SC_IT] == 0.0;
-  C c1, c2;
-  if (MODE == GS_P) {
-    c1 = mk(Real(be.x), Real(be.y));
-    const double2 bo = zmul(be, om);
-    c2 = mk(Real(-bo.x), Real(-bo.y));
-  } else if (MODE == GS_S) {
-    c2 = mk(Real(-al.x), Real(-al.y));
-  } else if (MODE == GS_X) {
-    c1 = mk(Real(al.x), Real(al.y));
-    c2 = mk(Real(om.x), Real(om.y));
-  } else {
-    c2 = mk(Real(-om.x), Real(-om.y));
-  }
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    C r;
-    if (MODE == GS_P) r = first ? A[i] : cadd(A[i], cadd(cmul(o[i], c1), cmul(Cc[i], c2)));
-    else if (MODE == GS_X) r = cadd(o[i], cadd(cmul(A[i], c1), cmul(Cc[i], c2)));
-    else r = cadd(A[i], cmul(Cc[i], c2));
-    o[i] = r;
-  }
+  pass_prologue();
+  __shared__ double red[3 * 256];
+  double acc[3] = {0, 0, 0};
+  const bool done = sc[SC_DONE] != 0.0;
+  const double2 al = gs_ld2(sc + SC_ALPHA), om = gs_ld2(sc + SC_OM);
+  const C a = mk(Real(al.x), Real(al.y)), w = mk(Real(om.x), Real(om.y));
+  if (!done)
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+      const C si = s[i], pi = p[i], ti = t[i], hi = rh[i];
+      C xi = x[i];
+      xi = mk(xi.x + a.x * pi.x - a.y * pi.y + w.x * si.x - w.y * si.y, xi.y + a.x * pi.y + a.y * pi.x + w.x * si.y + w.y * si.x);
+      const C ri = mk(si.x - w.x * ti.x + w.y * ti.y, si.y - w.x * ti.y - w.y * ti.x);
+      x[i] = xi;
+      r[i] = ri;
+      acc[0] += (double)hi.x * ri.x + (double)hi.y * ri.y;
+      acc[1] += (double)hi.x * ri.y - (double)hi.y * ri.x;
+      acc[2] += (double)ri.x * ri.x + (double)ri.y * ri.y;
+    }
+  block_sums(acc, red, [&](int v, double z) { part[(long long)v * stride + blockIdx.x] = z; });
 }
 
 // Spectral translation by x0 (the Nyquist mode takes cos(k_N x0), the mean of
@@ -394,15 +330,22 @@ fse_status shift_kick(fse_plan* P, void* psi, const double* x0, const double* kv
 
 size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// workspace: 10 complex fields, 3 real fields, reduction partials and results
+// partials per value: one per tile of the x passes or block of the vector kernels
+int gs_parts(const fse_plan* P) {
+  const int t = x_tiles(const_cast<fse_plan*>(P), P->ny * (P->dim == 3 ? P->nz : 1));
+  return t > kGsBlocks ? t : kGsBlocks;
+}
+
+// workspace: 8 complex fields (the last one only used with rotation), 3 real
+// fields, reduction partials and results
 struct GsLayout {
-  size_t cplx[10], real[3], part, out, sc, total;
+  size_t cplx[8], real[3], part, out, sc, total;
 };
 GsLayout gs_layout(const fse_plan* P) {
   GsLayout L;
   const size_t N = (size_t)P->nx * P->ny * P->nz;
   size_t off = 0;
-  for (int i = 0; i < 10; ++i) {
+  for (int i = 0; i < 8; ++i) {
     L.cplx[i] = off;
     off = al256(off + N * P->csize);
   }
@@ -411,7 +354,7 @@ GsLayout gs_layout(const fse_plan* P) {
     off = al256(off + N * P->rsize);
   }
   L.part = off;
-  off = al256(off + sizeof(double) * 4 * kGsBlocks);
+  off = al256(off + sizeof(double) * 4 * gs_parts(P));
   L.out = off;
   off = al256(off + sizeof(double) * 8);
   L.sc = off;
@@ -426,89 +369,122 @@ struct Gs {
   fse_plan* P;
   cudaStream_t st;
   long long N;
-  int blocks;
+  int blocks, nlines, tiles, stride;
   GsGrid g;
-  C *phin, *r, *rh, *p, *v, *s, *t, *t1, *t2, *t3;
+  C *phin, *r, *rh, *p, *v, *s, *t, *w;  // w: the operator's work field; phin doubles as d_y u inside a product
+  C* dy;
   Real *W, *pk, *Phi;
   double *part, *out, *sc;
   double omega;
 
-  fse_status chk(const char* w) { return launched(P, cudaGetLastError(), w); }
-
+  fse_status chk(const char* w0) { return launched(P, cudaGetLastError(), w0); }
   fse_status copy(C* dst, const C* src) {
     cudaError_t e = cudaMemcpyAsync(dst, src, (size_t)N * sizeof(C), cudaMemcpyDeviceToDevice, st);
     return e == cudaSuccess ? FSE_OK : cuda_fail(P, e, "ground state copy");
   }
-  fse_status lincomb(C* o, const C* A, std::complex<double> a, const C* B = nullptr,
-                     std::complex<double> b = 0.0, const C* Cc = nullptr, std::complex<double> c = 0.0) {
-    k_gs_lincomb<Real><<<blocks, 256, 0, st>>>(o, A, make_double2(a.real(), a.imag()), B,
-                                               make_double2(b.real(), b.imag()), Cc, make_double2(c.real(), c.imag()), N);
-    return chk("ground state update");
+  template <int MODE> fse_status fin(int count, int nv, double tol = 0.0) {
+    return launched(P, launch_pass(k_gs_fin<MODE>, 1, 256, 0, st, (const double*)part, stride, count, nv, out, sc, tol),
+                    "ground state reduction");
   }
-  // two complex inner products sum conj(a) b, read back to the host (synchronises)
-  fse_status dot2(const C* a1, const C* b1, const C* a2, const C* b2, std::complex<double>& d1,
-                  std::complex<double>& d2) {
-    k_gs_dot2<Real><<<blocks, 256, 0, st>>>(a1, b1, a2, b2, N, part);
-    fse_status s0 = chk("ground state reduction");
-    if (s0 != FSE_OK) return s0;
-    k_gs_final<<<4, 256, 0, st>>>(part, blocks, 0, out);
-    if ((s0 = chk("ground state reduction")) != FSE_OK) return s0;
-    double h[4];
-    cudaError_t e = cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(P, e, "ground state reduction");
-    d1 = std::complex<double>(h[0], h[1]);
-    d2 = std::complex<double>(h[2], h[3]);
-    return FSE_OK;
-  }
-  // the same two inner products into out[0..3], left on the device
-  fse_status dot2_dev(const C* a1, const C* b1, const C* a2, const C* b2) {
-    k_gs_dot2<Real><<<blocks, 256, 0, st>>>(a1, b1, a2, b2, N, part);
-    fse_status s0 = chk("ground state reduction");
-    if (s0 != FSE_OK) return s0;
-    k_gs_final<<<4, 256, 0, st>>>(part, blocks, 0, out);
-    return chk("ground state reduction");
-  }
-  template <int MODE> fse_status update(C* o, const C* A, const C* Cc) {
-    k_gs_update<Real, MODE><<<blocks, 256, 0, st>>>(o, A, Cc, sc, N);
-    return chk("ground state update");
-  }
-  fse_status maxdiff(const C* a, const C* b, double& m) {
-    k_gs_maxdiff<Real><<<blocks, 256, 0, st>>>(a, b, N, part);
-    fse_status s0 = chk("ground state reduction");
-    if (s0 != FSE_OK) return s0;
-    k_gs_final<<<1, 256, 0, st>>>(part, blocks, 1, out);
-    if ((s0 = chk("ground state reduction")) != FSE_OK) return s0;
-    cudaError_t e = cudaMemcpyAsync(&m, out, sizeof(double), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    return e == cudaSuccess ? FSE_OK : cuda_fail(P, e, "ground state reduction");
-  }
-  // y = (I + P_Delta A_TF) u   (u and y distinct; t1..t3 scratch)
-  fse_status matvec(const C* u, C* y) {
-    fse_status s0;
-    if ((s0 = copy(t1, u)) != FSE_OK) return s0;
-    if (omega != 0.0) {
-      if ((s0 = fft_full<Real>(P, t1, -1)) != FSE_OK) return s0;
-      const double inv_n = 1.0 / (double)N;
-      k_gs_ik<Real><<<blocks, 256, 0, st>>>(t1, t2, g, 0, inv_n);
-      if ((s0 = chk("ground state derivative")) != FSE_OK) return s0;
-      k_gs_ik<Real><<<blocks, 256, 0, st>>>(t1, t3, g, 1, inv_n);
-      if ((s0 = chk("ground state derivative")) != FSE_OK) return s0;
-      if ((s0 = fft_full<Real>(P, t2, +1)) != FSE_OK) return s0;
-      if ((s0 = fft_full<Real>(P, t3, +1)) != FSE_OK) return s0;
+  // the passes along y (and z) of P_Delta on the x-spectrum in w
+  fse_status precond_yz() {
+    MulArgs m;
+    std::memset(&m, 0, sizeof(m));
+    m.kin = pk;
+    m.lx = P->nx;
+    ColArgs ay{w, (long long)P->nx * P->ny, P->nx, P->nz, P->nx};
+    if (P->dim == 2) {
+      m.kin_sr = P->nx / 2 + 1;
+      return col(P, FSE_PASS_OTHER, P->ny, COL_RMUL, ay, m);
     }
-    k_gs_atf<Real><<<blocks, 256, 0, st>>>(u, t2, t3, W, t1, g, omega);
-    if ((s0 = chk("ground state operator")) != FSE_OK) return s0;
-    if ((s0 = precond(t1)) != FSE_OK) return s0;
-    return lincomb(y, u, 1.0, t1, 1.0);
-  }
-  // w <- P_Delta w (in place)
-  fse_status precond(C* w) {
     fse_status s0;
-    if ((s0 = fft_full<Real>(P, w, -1)) != FSE_OK) return s0;
-    k_gs_scale_real<Real><<<blocks, 256, 0, st>>>(w, pk, N);
-    if ((s0 = chk("ground state preconditioner")) != FSE_OK) return s0;
-    return fft_full<Real>(P, w, +1);
+    if ((s0 = col(P, FSE_PASS_OTHER, P->ny, COL_FWD, ay, m)) != FSE_OK) return s0;
+    m.lp = P->ny;
+    m.kin_sp = P->nx / 2 + 1;
+    m.kin_sr = (long long)(P->nx / 2 + 1) * (P->ny / 2 + 1);
+    ColArgs az{w, P->nx, (long long)P->nx * P->ny, P->ny, P->nx};
+    if ((s0 = col(P, FSE_PASS_OTHER, P->nz, COL_RMUL, az, m)) != FSE_OK) return s0;
+    return col(P, FSE_PASS_OTHER, P->ny, COL_INV, ay, m);
+  }
+  // d_y of u into dy (rotation)
+  fse_status deriv_y(const C* u) {
+    MulArgs m;
+    std::memset(&m, 0, sizeof(m));
+    m.dkr = g.dk[1] / P->ny;
+    ColArgs a{const_cast<C*>(u), (long long)P->nx * P->ny, P->nx, P->nz, P->nx};
+    a.out = dy;
+    return col(P, FSE_PASS_OTHER, P->ny, COL_DY, a, m);
+  }
+  // w = x-spectrum of A_TF u (or scale u), u by `mode` from a, c, o; with
+  // rotation u itself has to exist before its derivative along y is taken
+  fse_status fwd(int mode, const C* a, const C* c, C* o, const Real* Wf, double scale) {
+    GsFwd f;
+    std::memset(&f, 0, sizeof(f));
+    f.mode = mode;
+    f.nlines = nlines;
+    f.ny = P->ny;
+    f.a = a;
+    f.c = c;
+    f.o = o;
+    f.W = Wf;
+    f.scale = scale;
+    f.omega = omega;
+    f.lo0 = g.lo[0];
+    f.h0 = g.h[0];
+    f.lo1 = g.lo[1];
+    f.h1 = g.h[1];
+    f.dkx = g.dk[0];
+    f.sc = sc;
+    f.out = w;
+    fse_status s0;
+    if (omega != 0.0 && Wf) {
+      const C* u = a;
+      if (mode != U_PLAIN) {
+        // u into o (its x-spectrum, also computed, is overwritten below)
+        f.W = nullptr;
+        if ((s0 = launched(P, launch_gs_fwd<Real>(P->nx, f, twiddle(P, P->nx), st), "ground state update")) != FSE_OK)
+          return s0;
+        u = o;
+        f.mode = U_PLAIN;
+        f.a = o;
+        f.W = Wf;
+      }
+      if ((s0 = deriv_y(u)) != FSE_OK) return s0;
+      f.dy = dy;
+    }
+    return launched(P, launch_gs_fwd<Real>(P->nx, f, twiddle(P, P->nx), st), "ground state operator");
+  }
+  fse_status inv(int mode, const C* u, const C* q, C* y, C* y2) {
+    GsInv f;
+    f.mode = mode;
+    f.nlines = nlines;
+    f.in = w;
+    f.u = u;
+    f.q = q;
+    f.y = y;
+    f.y2 = y2;
+    f.part = part;
+    f.stride = stride;
+    return launched(P, launch_gs_inv<Real>(P->nx, f, twiddle(P, P->nx), st), "ground state operator");
+  }
+  // ||x||^2 / hd into out[0]
+  fse_status norm(const C* x) {
+    k_gs_norm<Real><<<blocks, 256, 0, st>>>(x, N, part);
+    fse_status s0 = chk("ground state reduction");
+    return s0 != FSE_OK ? s0 : fin<FIN_SUM>(blocks, 1);
+  }
+  // x <- x / ||x|| (norm in out[0]); with old also max |x - old| into out[1]
+  fse_status normalise(C* x, const C* old, double hd) {
+    k_gs_normalise<Real><<<blocks, 256, 0, st>>>(x, old, out, hd, N, part);
+    fse_status s0 = chk("ground state normalisation");
+    if (s0 != FSE_OK || !old) return s0;
+    return launched(P, launch_pass(k_gs_fin<FIN_MAX>, 1, 256, 0, st, (const double*)part, stride, blocks, 1, out + 1, sc, 0.0),
+                    "ground state reduction");
+  }
+  fse_status read(double* h, const double* d, int n) {
+    cudaError_t e = cudaMemcpyAsync(h, d, sizeof(double) * n, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    return e == cudaSuccess ? FSE_OK : cuda_fail(P, e, "ground state read");
   }
 };
 
@@ -521,10 +497,14 @@ fse_status ground_state(fse_plan* P, void* psi_v, void* ws, const fse_gs_opts& o
   G.P = P;
   G.st = P->stream;
   G.N = (long long)P->nx * P->ny * P->nz;
-  G.blocks = (int)std::min<long long>(kGsBlocks, (G.N + 255) / 256);
+  G.blocks = (int)std::min<long long>(2 * kSMs, (G.N + 255) / 256);
+  G.nlines = P->ny * (P->dim == 3 ? P->nz : 1);
+  G.tiles = x_tiles(P, G.nlines);
+  G.stride = gs_parts(P);
   G.g = gs_grid(P);
-  C** cp[10] = {&G.phin, &G.r, &G.rh, &G.p, &G.v, &G.s, &G.t, &G.t1, &G.t2, &G.t3};
-  for (int i = 0; i < 10; ++i) *cp[i] = reinterpret_cast<C*>(base + L.cplx[i]);
+  C** cp[8] = {&G.phin, &G.r, &G.rh, &G.p, &G.v, &G.s, &G.t, &G.dy};
+  for (int i = 0; i < 8; ++i) *cp[i] = reinterpret_cast<C*>(base + L.cplx[i]);
+  G.w = static_cast<C*>(P->ws_ptr(P->off_tmp));  // the plan's scratch field
   G.W = reinterpret_cast<Real*>(base + L.real[0]);
   G.pk = reinterpret_cast<Real*>(base + L.real[1]);
   G.Phi = reinterpret_cast<Real*>(base + L.real[2]);
@@ -536,67 +516,33 @@ fse_status ground_state(fse_plan* P, void* psi_v, void* ws, const fse_gs_opts& o
   const double hd = P->h[0] * P->h[1] * (P->dim == 3 ? P->h[2] : 1.0);
   const bool nl = has_nonlocal(P);
   fse_status st;
+  double h2[2];
 
   k_gs_precond_table<Real><<<G.blocks, 256, 0, G.st>>>(G.pk, G.g, 1.0 / o.dt, P->p.s, P->p.m * P->p.m,
                                                        1.0 / (double)G.N);
   if ((st = G.chk("ground state preconditioner")) != FSE_OK) return st;
-  std::complex<double> m2, dummy;
-  if ((st = G.dot2(x, x, x, x, m2, dummy)) != FSE_OK) return st;
-  if (!(m2.real() > 0.0)) return fail(P, FSE_ERR_INVALID, "ground state: zero initial field");
-  if ((st = G.lincomb(x, x, 1.0 / std::sqrt(hd * m2.real()))) != FSE_OK) return st;
+  if ((st = G.norm(x)) != FSE_OK || (st = G.read(h2, G.out, 1)) != FSE_OK) return st;
+  if (!(h2[0] > 0.0)) return fail(P, FSE_ERR_INVALID, "ground state: zero initial field");
+  if ((st = G.normalise(x, nullptr, hd)) != FSE_OK) return st;
 
   const double3 g2 = make_double3(0.5 * P->p.gamma[0] * P->p.gamma[0], 0.5 * P->p.gamma[1] * P->p.gamma[1],
                                   P->dim == 3 ? 0.5 * P->p.gamma[2] * P->p.gamma[2] : 0.0);
   const double3 lk = make_double3(P->p.lat_k[0], P->p.lat_k[1], P->dim == 3 ? P->p.lat_k[2] : 0.0);
-  // one BiCGStab iteration: every operand and coefficient is on the device, so
-  // the launches are captured once per call as a CUDA graph and replayed
+  // one BiCGStab iteration: every operand and coefficient is on the device
   auto iteration = [&]() -> fse_status {
     fse_status s0;
-    if ((s0 = G.template update<GS_P>(G.p, G.r, G.v)) != FSE_OK) return s0;
-    if ((s0 = G.matvec(G.p, G.v)) != FSE_OK) return s0;
-    if ((s0 = G.dot2_dev(G.rh, G.v, G.rh, G.v)) != FSE_OK) return s0;
-    k_gs_sc_alpha<<<1, 1, 0, G.st>>>(G.sc, G.out);
-    if ((s0 = G.chk("ground state scalars")) != FSE_OK) return s0;
-    if ((s0 = G.template update<GS_S>(G.s, G.r, G.v)) != FSE_OK) return s0;
-    if ((s0 = G.matvec(G.s, G.t)) != FSE_OK) return s0;
-    if ((s0 = G.dot2_dev(G.t, G.s, G.t, G.t)) != FSE_OK) return s0;
-    k_gs_sc_omega<<<1, 1, 0, G.st>>>(G.sc, G.out);
-    if ((s0 = G.chk("ground state scalars")) != FSE_OK) return s0;
-    if ((s0 = G.template update<GS_X>(x, G.p, G.s)) != FSE_OK) return s0;
-    if ((s0 = G.template update<GS_R>(G.r, G.s, G.t)) != FSE_OK) return s0;
-    if ((s0 = G.dot2_dev(G.rh, G.r, G.r, G.r)) != FSE_OK) return s0;
-    k_gs_sc_rho<<<1, 1, 0, G.st>>>(G.sc, G.out);
-    return G.chk("ground state scalars");
+    if ((s0 = G.fwd(U_P, G.r, G.v, G.p, G.W, 0.0)) != FSE_OK || (s0 = G.precond_yz()) != FSE_OK ||
+        (s0 = G.inv(V_ADD, G.p, G.rh, G.v, nullptr)) != FSE_OK || (s0 = G.template fin<FIN_ALPHA>(G.tiles, 2)) != FSE_OK)
+      return s0;
+    if ((s0 = G.fwd(U_S, G.r, G.v, G.s, G.W, 0.0)) != FSE_OK || (s0 = G.precond_yz()) != FSE_OK ||
+        (s0 = G.inv(V_ADD2, G.s, nullptr, G.t, nullptr)) != FSE_OK ||
+        (s0 = G.template fin<FIN_OMEGA>(G.tiles, 3)) != FSE_OK)
+      return s0;
+    s0 = launched(P, launch_pass(k_gs_update<Real>, G.blocks, 256, 0, G.st, x, G.r, (const C*)G.p, (const C*)G.s,
+                                 (const C*)G.t, (const C*)G.rh, (const double*)G.sc, G.N, G.part, G.stride),
+                  "ground state update");
+    return s0 != FSE_OK ? s0 : G.template fin<FIN_RHO>(G.blocks, 3);
   };
-  cudaGraphExec_t iter_exec = nullptr;
-  long long iter_launches = 0;
-  if (o.max_inner > 0 && o.max_outer > 0) {
-    // capture on the solve's own stream; if capture is refused (e.g. the
-    // thread is capturing another stream) the iterations are launched directly
-    const long long l0 = P->launches;
-    if (cudaStreamBeginCapture(G.st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-      const fse_status sq = iteration();
-      cudaGraph_t graph = nullptr;
-      const cudaError_t e = cudaStreamEndCapture(G.st, &graph);
-      if (sq != FSE_OK || e != cudaSuccess) {
-        if (graph) cudaGraphDestroy(graph);
-        return sq != FSE_OK ? sq : cuda_fail(P, e, "ground state capture");
-      }
-      const cudaError_t ei = cudaGraphInstantiate(&iter_exec, graph, 0);
-      cudaGraphDestroy(graph);
-      if (ei != cudaSuccess) return cuda_fail(P, ei, "ground state capture");
-      iter_launches = P->launches - l0;
-      P->launches = l0;
-    } else {
-      cudaGetLastError();
-    }
-  }
-  struct ExecGuard {
-    cudaGraphExec_t* e;
-    ~ExecGuard() {
-      if (*e) cudaGraphExecDestroy(*e);
-    }
-  } exec_guard{&iter_exec};
   int outer = 0;
   long long inner = 0;
   double change = 0.0, res = 0.0;
@@ -607,14 +553,13 @@ fse_status ground_state(fse_plan* P, void* psi_v, void* ws, const fse_gs_opts& o
                                                       P->p.lat_amp, lk);
     if ((st = G.chk("ground state potential")) != FSE_OK) return st;
     // b = P_Delta phi^n / dt (held in s), r = b - M x, rh = r
-    if ((st = G.lincomb(G.s, G.phin, 1.0 / o.dt)) != FSE_OK) return st;
-    if ((st = G.precond(G.s)) != FSE_OK) return st;
-    if ((st = G.matvec(x, G.v)) != FSE_OK) return st;
-    if ((st = G.lincomb(G.r, G.s, 1.0, G.v, -1.0)) != FSE_OK) return st;
-    if ((st = G.copy(G.rh, G.r)) != FSE_OK) return st;
-    if ((st = G.dot2_dev(G.s, G.s, G.r, G.r)) != FSE_OK) return st;
-    k_gs_sc_init<<<1, 1, 0, G.st>>>(G.sc, G.out, o.inner_tol);
-    if ((st = G.chk("ground state scalars")) != FSE_OK) return st;
+    if ((st = G.fwd(U_PLAIN, x, nullptr, nullptr, nullptr, 1.0 / o.dt)) != FSE_OK || (st = G.precond_yz()) != FSE_OK ||
+        (st = G.inv(V_SET, nullptr, nullptr, G.s, nullptr)) != FSE_OK)
+      return st;
+    if ((st = G.fwd(U_PLAIN, x, nullptr, nullptr, G.W, 0.0)) != FSE_OK || (st = G.precond_yz()) != FSE_OK ||
+        (st = G.inv(V_RES, x, G.s, G.r, G.rh)) != FSE_OK ||
+        (st = G.template fin<FIN_INIT>(G.tiles, 3, o.inner_tol)) != FSE_OK)
+      return st;
     // Iterations are queued one ahead of the host: after queueing iteration
     // it, the host waits for the scalars of iteration it - 1 (copied to pinned
     // host memory behind it) and stops once they say done, so the GPU never
@@ -622,13 +567,7 @@ fse_status ground_state(fse_plan* P, void* psi_v, void* ws, const fse_gs_opts& o
     double* hs = P->gs_host;
     int it = 0;
     for (; it < o.max_inner; ++it) {
-      if (iter_exec) {
-        cudaError_t e = cudaGraphLaunch(iter_exec, G.st);
-        if (e != cudaSuccess) return cuda_fail(P, e, "ground state iteration");
-        P->launches += iter_launches;
-      } else if ((st = iteration()) != FSE_OK) {
-        return st;
-      }
+      if ((st = iteration()) != FSE_OK) return st;
       cudaError_t e = cudaMemcpyAsync(hs + (it & 1) * SC_SIZE, G.sc, sizeof(double) * SC_SIZE,
                                       cudaMemcpyDeviceToHost, G.st);
       if (e == cudaSuccess) e = cudaEventRecord(P->gs_ev[it & 1], G.st);
@@ -639,21 +578,16 @@ fse_status ground_state(fse_plan* P, void* psi_v, void* ws, const fse_gs_opts& o
         if (hs[((it - 1) & 1) * SC_SIZE + SC_DONE] != 0.0) break;
       }
     }
-    // the scalars after the last queued iteration (iteration count, residual)
-    {
-      cudaError_t e = cudaMemcpyAsync(hs, G.sc, sizeof(double) * SC_SIZE, cudaMemcpyDeviceToHost, G.st);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(G.st);
-      if (e != cudaSuccess) return cuda_fail(P, e, "ground state scalars");
-    }
-    it = (int)hs[SC_IT];
+    // phi^{n+1} = phi^(1) / ||phi^(1)||, and max |phi^{n+1} - phi^n|; then one
+    // read of the scalars after the last queued iteration, the norm and the change
+    if ((st = G.norm(x)) != FSE_OK || (st = G.normalise(x, G.phin, hd)) != FSE_OK) return st;
+    cudaError_t e = cudaMemcpyAsync(hs, G.sc, sizeof(double) * SC_SIZE, cudaMemcpyDeviceToHost, G.st);
+    if (e != cudaSuccess) return cuda_fail(P, e, "ground state scalars");
+    if ((st = G.read(h2, G.out, 2)) != FSE_OK) return st;
     res = hs[SC_RES];
-    inner += it;
-    // phi^{n+1} = phi^(1) / ||phi^(1)||
-    if ((st = G.dot2(x, x, x, x, m2, dummy)) != FSE_OK) return st;
-    if (!(m2.real() > 0.0)) return fail(P, FSE_ERR_NONFINITE, "ground state: zero field");
-    if ((st = G.lincomb(x, x, 1.0 / std::sqrt(hd * m2.real()))) != FSE_OK) return st;
-    if ((st = G.maxdiff(x, G.phin, change)) != FSE_OK) return st;
-    change /= o.dt;
+    inner += (int)hs[SC_IT];
+    if (!(h2[0] > 0.0)) return fail(P, FSE_ERR_NONFINITE, "ground state: zero field");
+    change = h2[1] / o.dt;
     ++outer;
     if (!std::isfinite(change)) return fail(P, FSE_ERR_NONFINITE, "ground state: non-finite iterate");
     if (change <= o.tol) break;

@@ -66,6 +66,7 @@ const double kPi = 3.14159265358979323846;
 fse_status fail(fse_plan* p, fse_status st, const std::string& msg);
 fse_status cuda_fail(fse_plan* p, cudaError_t e, const char* where);
 fse_status launched(fse_plan* P, cudaError_t e, const char* where);
+const void* twiddle(const fse_plan* P, int L);
 cudaEvent_t prof_begin(fse_plan* P);
 void prof_end(fse_plan* P, int kind, cudaEvent_t a);
 fse_status col(fse_plan* P, int kind, int n, int var, const ColArgs& a, const MulArgs& m);

@@ -14,7 +14,7 @@ namespace fse {
 // Launch of a step pass with programmatic dependent launch on the previous
 // kernel in the stream (see pass_prologue).
 template <typename... Params, typename... Args>
-static cudaError_t launch_pass(void (*kernel)(Params...), unsigned blocks, unsigned threads, size_t smem,
+static cudaError_t launch_pass_if(bool pdl, void (*kernel)(Params...), unsigned blocks, unsigned threads, size_t smem,
                                cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks);
@@ -23,10 +23,23 @@ static cudaError_t launch_pass(void (*kernel)(Params...), unsigned blocks, unsig
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = pdl;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... Params, typename... Args>
+static cudaError_t launch_pass(void (*kernel)(Params...), unsigned blocks, unsigned threads, size_t smem,
+                               cudaStream_t st, Args... args) {
+  return launch_pass_if(true, kernel, blocks, threads, smem, st, args...);
+}
+
+// A float64 pass of one to four tiles per SM is not launched early: its blocks
+// would be dealt to the SMs while the previous pass's still sit there unevenly,
+// and the SM that gets one too many sets the time of a pass bound by the FP64
+// pipe (ground state on 512^2: inverse x pass 47 us early, 25 us after).
+template <typename Real> static bool launch_early(long long blocks) {
+  return sizeof(Real) == 4 || blocks < kSMs || blocks >= 4 * kSMs;
 }
 
 // cudaFuncSetAttribute once per kernel and device when the dynamic tile comes
@@ -54,9 +67,10 @@ static cudaError_t col_launch(const ColArgs& a, const MulArgs& m, long long bloc
   if (e != cudaSuccess) return e;
   if (blocks <= 0) return cudaSuccess;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+  if (a.blocks_out) *a.blocks_out = (int)blocks;
   MulArgs mf = m;
   fill_f32(mf);
-  return launch_pass(k_col<Real, N, VAR, NP>, (unsigned)blocks, K::NT, K::smem(), st, a, mf,
+  return launch_pass_if(launch_early<Real>(blocks), k_col<Real, N, VAR, NP>, (unsigned)blocks, K::NT, K::smem(), st, a, mf,
                      reinterpret_cast<const C*>(tw));
 }
 
@@ -109,7 +123,7 @@ static cudaError_t x_launch(const XArgs& a, const void* twn, const void* tw2n, c
   if (blocks <= 0) return cudaSuccess;
   XArgs af = a;
   fill_f32(af);
-  return launch_pass(k_xpass<Real, NX, LN, KIND>, (unsigned)blocks, K::NT, K::smem(), st, af,
+  return launch_pass_if(launch_early<Real>(blocks), k_xpass<Real, NX, LN, KIND>, (unsigned)blocks, K::NT, K::smem(), st, af,
                      reinterpret_cast<const C*>(twn), reinterpret_cast<const C*>(tw2n));
 }
 

@@ -29,108 +29,81 @@ constexpr int kPartStride = 65536;  // partials per slot (>= x-pass blocks of th
 constexpr int kRedBlocks = 1024;
 
 struct ObsArgs {
-  int nx, ny, nz;
+  int nx, ny, nlines;
   double lo[3], h[3];
-  double g2[3];  // gamma_v^2 / 2
   double c, s;   // cos, sin of Omega t
   double lat_amp, lat_k[3];  // optical lattice lat_amp sum_v sin^2(lat_k[v] x_v)
 };
 
+// Moments of the density in float64, one warp per line, in index units from
+// the grid's middle (exact): along a line only the sums of rho, rho^2, rho i
+// and rho i^2 are formed, and a line's y and z enter once; the coordinates and
+// the harmonic trap energy follow from the sums on the host. About 13 float64
+// slots per point in place of 45 (128^3: 172 -> 50 us, the FP64 pipe's time).
+// Slots: rho, rho^2, lattice energy, and rho times i, j, k, i i, j j, k k, i j.
 template <typename Real>
-__global__ void __launch_bounds__(256) k_obs_phys(const typename Cplx<Real>::T* __restrict__ psi, ObsArgs o,
+__global__ void __launch_bounds__(256) k_obs_phys(const typename Cplx<Real>::T* __restrict__ psi, ObsArgs o, int nz,
                                                   double* part) {
-  __shared__ double red[32];
-  const long long N = (long long)o.nx * o.ny * o.nz;
+  __shared__ double red[10 * 256];
+  const int lane = threadIdx.x & 31, nw = gridDim.x * 8;
   double acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const int ix = (int)(i % o.nx);
-    const long long r = i / o.nx;
-    const int iy = (int)(r % o.ny), iz = (int)(r / o.ny);
-    const double x = o.lo[0] + o.h[0] * ix, y = o.lo[1] + o.h[1] * iy, z = o.lo[2] + o.h[2] * iz;
-    const typename Cplx<Real>::T u = psi[i];
-    const double rho = (double)u.x * u.x + (double)u.y * u.y;
-    const double X = o.c * x + o.s * y, Y = -o.s * x + o.c * y;
-    double W = o.g2[0] * X * X + o.g2[1] * Y * Y + o.g2[2] * z * z;
-    if (o.lat_amp != 0.0) {
-      const double sx = sin(o.lat_k[0] * X), sy = sin(o.lat_k[1] * Y), sz = sin(o.lat_k[2] * z);
-      W += o.lat_amp * (sx * sx + sy * sy + sz * sz);
+  for (int l = blockIdx.x * 8 + (threadIdx.x >> 5); l < o.nlines; l += nw) {
+    const typename Cplx<Real>::T* row = psi + (long long)l * o.nx;
+    const int iy = l % o.ny, iz = l / o.ny;
+    double s0 = 0.0, s1 = 0.0, i0 = lane - o.nx / 2;
+#pragma unroll 4
+    for (int x = lane; x < o.nx; x += 32, i0 += 32.0) {
+      const typename Cplx<Real>::T u = row[x];
+      const double rho = (double)u.x * u.x + (double)u.y * u.y, t = rho * i0;
+      s0 += rho;
+      acc[1] = fma(rho, rho, acc[1]);
+      s1 += t;
+      acc[6] = fma(t, i0, acc[6]);
     }
-    acc[0] += rho;
-    acc[1] += rho * rho;
-    acc[2] += W * rho;
-    acc[3] += x * rho;
-    acc[4] += y * rho;
-    acc[5] += z * rho;
-    acc[6] += x * x * rho;
-    acc[7] += y * y * rho;
-    acc[8] += z * z * rho;
-    acc[9] += x * y * rho;
+    if (o.lat_amp != 0.0) {
+      const double y = o.lo[1] + o.h[1] * iy, z = o.lo[2] + o.h[2] * iz;
+      for (int x = lane; x < o.nx; x += 32) {
+        const typename Cplx<Real>::T u = row[x];
+        const double rho = (double)u.x * u.x + (double)u.y * u.y, xx = o.lo[0] + o.h[0] * x;
+        const double sx = sin(o.lat_k[0] * (o.c * xx + o.s * y)), sy = sin(o.lat_k[1] * (-o.s * xx + o.c * y)),
+                     sz = sin(o.lat_k[2] * z);
+        acc[2] += o.lat_amp * (sx * sx + sy * sy + sz * sz) * rho;
+      }
+    }
+    const double j = iy - o.ny / 2, k = iz - nz / 2, a = j * s0, b = k * s0;
+    acc[0] += s0;
+    acc[3] += s1;
+    acc[4] += a;
+    acc[5] += b;
+    acc[7] = fma(j, a, acc[7]);
+    acc[8] = fma(k, b, acc[8]);
+    acc[9] = fma(j, s1, acc[9]);
   }
-#pragma unroll
-  for (int k = 0; k < 10; ++k) {
-    const double v = block_sum(acc[k], red);
-    if (threadIdx.x == 0) part[k * kPartStride + blockIdx.x] = v;
-  }
+  block_sums(acc, red, [&](int k, double v) { part[k * kPartStride + blockIdx.x] = v; });
 }
 
-// sum over the spectrum of (|k|^2 + m^2)^s |phi^_k|^2 (unnormalised DFT)
+// sum over the spectrum of (|k|^2 + m^2)^s |phi^_k|^2 (unnormalised DFT), one warp per line
 template <typename Real>
-__global__ void __launch_bounds__(256) k_obs_kin(const typename Cplx<Real>::T* __restrict__ sp, ObsArgs o,
+__global__ void __launch_bounds__(256) k_obs_kin(const typename Cplx<Real>::T* __restrict__ sp, ObsArgs o, int nz,
                                                  double dkx, double dky, double dkz, double s, double m2,
                                                  double* part) {
   __shared__ double red[32];
-  const long long N = (long long)o.nx * o.ny * o.nz;
+  const int lane = threadIdx.x & 31, nw = gridDim.x * 8;
   double acc = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const int ix = (int)(i % o.nx);
-    const long long r = i / o.nx;
-    const int iy = (int)(r % o.ny), iz = (int)(r / o.ny);
-    const Real kx = Real(dkx) * Real(wrap_index(ix, o.nx));
-    const Real ky = Real(dky) * Real(wrap_index(iy, o.ny));
-    const Real kz = o.nz > 1 ? Real(dkz) * Real(wrap_index(iz, o.nz)) : Real(0);
-    const Real k2 = kx * kx + ky * ky + kz * kz + Real(m2);
-    const typename Cplx<Real>::T u = sp[i];
-    acc += (double)pow(k2, Real(s)) * ((double)u.x * u.x + (double)u.y * u.y);
+  for (int l = blockIdx.x * 8 + (threadIdx.x >> 5); l < o.nlines; l += nw) {
+    const typename Cplx<Real>::T* row = sp + (long long)l * o.nx;
+    const Real ky = Real(dky) * Real(wrap_index(l % o.ny, o.ny));
+    const Real kz = nz > 1 ? Real(dkz) * Real(wrap_index(l / o.ny, nz)) : Real(0);
+#pragma unroll 4
+    for (int x = lane; x < o.nx; x += 32) {
+      const Real kx = Real(dkx) * Real(wrap_index(x, o.nx));
+      const Real k2 = kx * kx + ky * ky + kz * kz + Real(m2);
+      const typename Cplx<Real>::T u = row[x];
+      acc += (double)pow(k2, Real(s)) * ((double)u.x * u.x + (double)u.y * u.y);
+    }
   }
   const double v = block_sum(acc, red);
   if (threadIdx.x == 0) part[SL_KIN * kPartStride + blockIdx.x] = v;
-}
-
-// d = i k_axis phi^ / N (odd factor zero at the Nyquist index)
-template <typename Real>
-__global__ void __launch_bounds__(256) k_mul_ik(const typename Cplx<Real>::T* __restrict__ sp,
-                                                typename Cplx<Real>::T* __restrict__ d, ObsArgs o, int axis,
-                                                double dk, double inv_n) {
-  const long long N = (long long)o.nx * o.ny * o.nz;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const int ix = (int)(i % o.nx);
-    const int iy = (int)((i / o.nx) % o.ny);
-    const int idx = axis == 0 ? ix : iy;
-    const int n = axis == 0 ? o.nx : o.ny;
-    const Real k = (2 * idx == n) ? Real(0) : Real(dk * inv_n) * Real(wrap_index(idx, n));
-    const typename Cplx<Real>::T u = sp[i];
-    d[i] = mk(-k * u.y, k * u.x);
-  }
-}
-
-// sum of c(x) Im(conj(psi) d): with c = x the y-derivative term, with c = -y the x-derivative term of
-// <psi, -i (x d_y - y d_x) psi>
-template <typename Real>
-__global__ void __launch_bounds__(256) k_obs_lz(const typename Cplx<Real>::T* __restrict__ psi,
-                                                const typename Cplx<Real>::T* __restrict__ d, ObsArgs o, int axis,
-                                                int slot, double* part) {
-  __shared__ double red[32];
-  const long long N = (long long)o.nx * o.ny * o.nz;
-  double acc = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const int ix = (int)(i % o.nx);
-    const int iy = (int)((i / o.nx) % o.ny);
-    const double c = axis == 1 ? (o.lo[0] + o.h[0] * ix) : -(o.lo[1] + o.h[1] * iy);
-    const typename Cplx<Real>::T u = psi[i], v = d[i];
-    acc += c * ((double)u.x * v.y - (double)u.y * v.x);
-  }
-  const double v = block_sum(acc, red);
-  if (threadIdx.x == 0) part[slot * kPartStride + blockIdx.x] = v;
 }
 
 struct SlotCounts {
@@ -234,20 +207,14 @@ template fse_status fft_full<float>(fse_plan*, void*, int);
 template fse_status fft_full<double>(fse_plan*, void*, int);
 
 fse_status nonlocal_field(fse_plan* P, const void* psi, const double* mdir, void* phi) {
-  void* tmp = P->ws_ptr(P->off_tmp);
   void* spec = P->ws_ptr(P->off_spec);
-  cudaError_t e;
   fse_status st;
-  if ((e = cudaMemcpyAsync(tmp, psi, P->psi_bytes, cudaMemcpyDeviceToDevice, P->stream)) != cudaSuccess)
-    return cuda_fail(P, e, "nonlocal field copy");
-  XArgs xa = x_args(P, tmp, spec);
-  if ((st = xpass(P, XP_FWD, xa)) != FSE_OK) return st;
-  if ((st = xpass(P, XP_E, xa)) != FSE_OK) return st;  // S = R2C of nx^2 rho
+  XArgs xa = x_args(P, const_cast<void*>(psi), spec);
+  if ((st = xpass(P, XP_D, xa)) != FSE_OK) return st;  // S = R2C of rho
   const double* md = mdir ? mdir : P->p.dip_n;
-  if ((st = nonlocal_yz(P, spec, 0.0, 0.0, false, md, 1.0 / ((double)P->nx * P->nx))) != FSE_OK) return st;
-  XArgs xr = x_args(P, const_cast<void*>(psi), spec);
-  xr.out = phi;
-  return xpass(P, XP_R, xr);
+  if ((st = nonlocal_yz(P, spec, 0.0, 0.0, false, md, 1.0)) != FSE_OK) return st;
+  xa.out = phi;
+  return xpass(P, XP_R, xa);
 }
 
 template <typename Real>
@@ -266,27 +233,25 @@ fse_status observables(fse_plan* P, const void* psi_in, double t, const double* 
   ObsArgs o;
   o.nx = P->nx;
   o.ny = P->ny;
-  o.nz = P->nz;
+  o.nlines = P->ny * P->nz;
+  double g2[3];  // gamma_v^2 / 2
   for (int j = 0; j < 3; ++j) {
     o.lo[j] = j < P->dim ? P->p.lo[j] : 0.0;
     o.h[j] = P->h[j];
     const double g = j < P->dim ? (gam ? gam[j] : P->p.gamma[j]) : 0.0;
-    o.g2[j] = 0.5 * g * g;
+    g2[j] = 0.5 * g * g;
     o.lat_k[j] = j < P->dim ? P->p.lat_k[j] : 0.0;
   }
   o.c = std::cos(P->p.omega * t);
   o.s = std::sin(P->p.omega * t);
   o.lat_amp = P->p.lat_amp;
   const long long N = (long long)P->nx * P->ny * P->nz;
-  const int blocks = (int)std::min<long long>(kRedBlocks, (N + 255) / 256);
+  const int blocks = std::min(2 * kSMs, (o.nlines + 7) / 8);
 
   // nonlocal energy density: Phi = U~(., t) * rho (un-integrated kernel at time t)
   if (has_nonlocal(P)) {
-    if ((e = cudaMemcpyAsync(tmp, psi, P->psi_bytes, cudaMemcpyDeviceToDevice, P->stream)) != cudaSuccess)
-      return cuda_fail(P, e, "observables copy");
-    XArgs xa = x_args(P, tmp, spec);
-    if ((st = xpass(P, XP_FWD, xa)) != FSE_OK) return st;
-    if ((st = xpass(P, XP_E, xa)) != FSE_OK) return st;  // tmp = nx psi, S = R2C of nx^2 rho
+    XArgs xr = x_args(P, const_cast<C*>(psi), spec);
+    if ((st = xpass(P, XP_D, xr)) != FSE_OK) return st;  // S = R2C of rho
     double mdir[3] = {0, 0, 0};
     if (P->p.kernel == FSE_KERNEL_DDI3D || P->p.kernel == FSE_KERNEL_DDI2D) {
       // m(t) = A(t)^T n
@@ -295,8 +260,7 @@ fse_status observables(fse_plan* P, const void* psi_in, double t, const double* 
       mdir[1] = o.s * n1 + o.c * n2;
       mdir[2] = n3;
     }
-    if ((st = nonlocal_yz(P, spec, t, t, false, mdir, 1.0 / ((double)P->nx * P->nx))) != FSE_OK) return st;
-    XArgs xr = x_args(P, const_cast<C*>(psi), spec);
+    if ((st = nonlocal_yz(P, spec, t, t, false, mdir, 1.0)) != FSE_OK) return st;
     xr.part = part + SL_NON * kPartStride;
     if (x_tiles(P, xr.nlines) > kPartStride) return fail(P, FSE_ERR_UNSUPPORTED, "observables: grid too large");
     if ((st = xpass(P, XP_R, xr)) != FSE_OK) return st;
@@ -304,38 +268,50 @@ fse_status observables(fse_plan* P, const void* psi_in, double t, const double* 
   }
 
   cudaEvent_t ev = prof_begin(P);
-  k_obs_phys<Real><<<blocks, 256, 0, P->stream>>>(psi, o, part);
+  k_obs_phys<Real><<<blocks, 256, 0, P->stream>>>(psi, o, P->nz, part);
   prof_end(P, FSE_PASS_OTHER, ev);
   if ((st = launched(P, cudaGetLastError(), "observables")) != FSE_OK) return st;
   for (int k = SL_MASS; k <= SL_XY; ++k) cnt.n[k] = blocks;
 
-  // spectrum of psi
-  if ((e = cudaMemcpyAsync(tmp, psi, P->psi_bytes, cudaMemcpyDeviceToDevice, P->stream)) != cudaSuccess)
-    return cuda_fail(P, e, "observables copy");
-  if ((st = fft_full<Real>(P, tmp, -1)) != FSE_OK) return st;
+  // spectrum of psi (in the scratch field)
   const double dkx = 2 * kPi / (P->p.hi[0] - P->p.lo[0]);
   const double dky = 2 * kPi / (P->p.hi[1] - P->p.lo[1]);
   const double dkz = P->dim == 3 ? 2 * kPi / (P->p.hi[2] - P->p.lo[2]) : 0.0;
+  MulArgs m;
+  std::memset(&m, 0, sizeof(m));
+  XArgs x0 = x_args(P, tmp, nullptr);
+  x0.aux = psi;
+  if ((st = xpass(P, XP_FWD, x0)) != FSE_OK) return st;
+  ColArgs ay{tmp, (long long)P->nx * P->ny, P->nx, P->nz, P->nx};
+  if ((st = col(P, FSE_PASS_OTHER, P->ny, COL_FWD, ay, m)) != FSE_OK) return st;
+  if (P->dim == 3) {
+    ColArgs az{tmp, P->nx, (long long)P->nx * P->ny, P->ny, P->nx};
+    if ((st = col(P, FSE_PASS_OTHER, P->nz, COL_FWD, az, m)) != FSE_OK) return st;
+  }
   ev = prof_begin(P);
-  k_obs_kin<Real><<<blocks, 256, 0, P->stream>>>(tmp, o, dkx, dky, dkz, P->p.s, P->p.m * P->p.m, part);
+  k_obs_kin<Real><<<blocks, 256, 0, P->stream>>>(tmp, o, P->nz, dkx, dky, dkz, P->p.s, P->p.m * P->p.m, part);
   prof_end(P, FSE_PASS_OTHER, ev);
   if ((st = launched(P, cudaGetLastError(), "observables")) != FSE_OK) return st;
   cnt.n[SL_KIN] = blocks;
 
-  // <L_z>: spectral derivatives d_y psi (paired with x) and d_x psi (paired with -y)
-  for (int axis = 1; axis >= 0; --axis) {
-    ev = prof_begin(P);
-    k_mul_ik<Real><<<blocks, 256, 0, P->stream>>>(tmp, spec, o, axis, axis == 0 ? dkx : dky, 1.0 / (double)N);
-    prof_end(P, FSE_PASS_OTHER, ev);
-    if ((st = launched(P, cudaGetLastError(), "observables")) != FSE_OK) return st;
-    if ((st = fft_full<Real>(P, spec, +1)) != FSE_OK) return st;
-    const int slot = axis == 1 ? SL_LZY : SL_LZX;
-    ev = prof_begin(P);
-    k_obs_lz<Real><<<blocks, 256, 0, P->stream>>>(psi, spec, o, axis, slot, part);
-    prof_end(P, FSE_PASS_OTHER, ev);
-    if ((st = launched(P, cudaGetLastError(), "observables")) != FSE_OK) return st;
-    cnt.n[slot] = blocks;
-  }
+  // <L_z> = Im sum conj(psi) (x d_y - y d_x) psi: each derivative needs the
+  // transforms of its own axis alone, and its product with psi is summed where
+  // it is formed
+  XArgs xl = x_args(P, const_cast<C*>(psi), nullptr);
+  xl.beta_dt = dkx / P->nx;
+  xl.part = part + SL_LZX * kPartStride;
+  if (x_tiles(P, xl.nlines) > kPartStride) return fail(P, FSE_ERR_UNSUPPORTED, "observables: grid too large");
+  if ((st = xpass(P, XP_LZ, xl)) != FSE_OK) return st;
+  cnt.n[SL_LZX] = x_tiles(P, xl.nlines);
+  m.dkr = dky / P->ny;
+  ColArgs al{const_cast<C*>(psi), (long long)P->nx * P->ny, P->nx, P->nz, P->nx};
+  al.part = part + SL_LZY * kPartStride;
+  al.lo = o.lo[0];
+  al.h = o.h[0];
+  int lz_blocks = 0;
+  al.blocks_out = &lz_blocks;
+  if ((st = col(P, FSE_PASS_OTHER, P->ny, COL_LZ, al, m)) != FSE_OK) return st;
+  cnt.n[SL_LZY] = lz_blocks;
 
   k_sum_slots<<<NSLOT, 256, 0, P->stream>>>(part, cnt, sums);
   if ((st = launched(P, cudaGetLastError(), "observables")) != FSE_OK) return st;
@@ -346,10 +322,24 @@ fse_status observables(fse_plan* P, const void* psi_in, double t, const double* 
 
   double hd = 1.0;
   for (int j = 0; j < P->dim; ++j) hd *= P->h[j];
+  // sums in index units from the middle -> coordinates x = c + h i
+  {
+    const int n3[3] = {P->nx, P->ny, P->nz};
+    double c[3];
+    for (int j = 0; j < 3; ++j) c[j] = j < P->dim ? o.lo[j] + o.h[j] * (n3[j] / 2) : 0.0;
+    const double s0 = h[SL_MASS], i1[3] = {h[SL_X], h[SL_Y], h[SL_Z]};
+    h[SL_XY] = c[0] * c[1] * s0 + c[0] * o.h[1] * i1[1] + c[1] * o.h[0] * i1[0] + o.h[0] * o.h[1] * h[SL_XY];
+    for (int j = 0; j < 3; ++j) {
+      h[SL_XX + j] = c[j] * c[j] * s0 + 2 * c[j] * o.h[j] * i1[j] + o.h[j] * o.h[j] * h[SL_XX + j];
+      h[SL_X + j] = c[j] * s0 + o.h[j] * i1[j];
+    }
+  }
   std::memset(out, 0, sizeof(*out));
   out->mass = hd * h[SL_MASS];
   out->e_kin = 0.5 * hd / (double)N * h[SL_KIN];
-  out->e_pot = hd * h[SL_WRHO];
+  // W = g2_x X^2 + g2_y Y^2 + g2_z z^2 (+ lattice), X = c x + s y, Y = -s x + c y
+  out->e_pot = hd * (h[SL_WRHO] + g2[0] * (o.c * o.c * h[SL_XX] + 2 * o.c * o.s * h[SL_XY] + o.s * o.s * h[SL_YY]) +
+                     g2[1] * (o.s * o.s * h[SL_XX] - 2 * o.c * o.s * h[SL_XY] + o.c * o.c * h[SL_YY]) + g2[2] * h[SL_ZZ]);
   out->e_int = 0.5 * P->p.beta * hd * h[SL_RHO2];
   out->e_non = has_nonlocal(P) ? 0.5 * P->p.lambda * hd * h[SL_NON] : 0.0;
   out->lz = hd * (h[SL_LZY] + h[SL_LZX]);

@@ -23,7 +23,7 @@
 
 namespace fse {
 
-enum { XP_FWD = 0, XP_INV = 1, XP_E = 2, XP_A = 3, XP_R = 4, XP_ADJ1 = 5, XP_ADJ2 = 6, XP_AL = 7 };
+enum { XP_FWD = 0, XP_INV = 1, XP_E = 2, XP_A = 3, XP_R = 4, XP_ADJ1 = 5, XP_ADJ2 = 6, XP_AL = 7, XP_D = 8, XP_LZ = 9 };
 
 struct XArgs {
   void* psi;
@@ -79,25 +79,6 @@ __host__ __device__ inline void fill_f32(XArgs& a) {
     a.f.lat_c[i] = (float)a.lat_c[i];
     a.f.lat_s[i] = (float)a.lat_s[i];
   }
-}
-
-// Deterministic float64 block sum (blockDim.x <= 1024; the last warp may be
-// partly filled); result in thread 0.
-__device__ __forceinline__ double block_sum(double v, double* sh) {
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-  const int lanes = min(32, (int)blockDim.x - 32 * w);
-  const unsigned mask = lanes == 32 ? 0xffffffffu : (1u << lanes) - 1u;
-  for (int o = 16; o > 0; o >>= 1) {
-    const double t = __shfl_down_sync(mask, v, o);
-    if (l + o < lanes) v += t;
-  }
-  __syncthreads();
-  if (l == 0) sh[w] = v;
-  __syncthreads();
-  v = 0.0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < nw; ++i) v += sh[i];
-  return v;
 }
 
 // Rounded products and fused multiply-adds that the compiler does not
@@ -509,11 +490,12 @@ __device__ __forceinline__ void xpass_body(const XArgs& a, const typename TwOf<R
     // a narrow tile is alone on its SM: its twiddle tables come into L1 before
     // the wait for the previous pass (see col_tile)
     unsigned x = 0;
-    if constexpr (F1::P.np > 1 && KIND != XP_R && KIND != XP_ADJ1 && KIND != XP_ADJ2)
+    if constexpr (KIND != XP_R && KIND != XP_ADJ1 && KIND != XP_ADJ2 && KIND != XP_D)
       x = F1::template warm_table<false, true, K::NT>(twn, tid);
     if constexpr (KIND != XP_FWD && KIND != XP_INV) {
-      if (KIND == XP_E || (KIND == XP_ADJ1 && a.use_spec)) x ^= F2::template warm_table<false, false, K::NT>(tw2n, tid);
-      if (KIND != XP_E && a.use_spec) x ^= F2::template warm_table<true, false, K::NT>(tw2n, tid);
+      if (KIND == XP_LZ) x ^= F1::template warm_table<true, true, K::NT>(twn, tid);
+      if (KIND == XP_E || KIND == XP_D || (KIND == XP_ADJ1 && a.use_spec)) x ^= F2::template warm_table<false, false, K::NT>(tw2n, tid);
+      if (KIND != XP_E && KIND != XP_D && KIND != XP_LZ && a.use_spec) x ^= F2::template warm_table<true, false, K::NT>(tw2n, tid);
     }
     reinterpret_cast<unsigned*>(smem_raw)[tid] = x;
   }
@@ -551,9 +533,41 @@ __device__ __forceinline__ void xpass_body(const XArgs& a, const typename TwOf<R
     __syncthreads();
   };
 
-  if constexpr (KIND == XP_FWD || KIND == XP_INV || KIND == XP_E) {
+  if constexpr (KIND == XP_D) {
+    // the density of psi itself (psi is only read)
+    F1::template each<F1::RF>(it, [&](int, int x, int) {
+      const Vec<L> u = line_ld<NX>((const C*)line0, g, nl, x);
+      real_st<RS>(field, g, x, lfma(u.re, u.re, lmul(u.im, u.im)));
+    });
+    __syncthreads();
+    r2c();
+  } else if constexpr (KIND == XP_LZ) {
+    // partial of -sum y Im(conj(psi) d_x psi), d_x by the line's own transforms (beta_dt: 2 pi / (W n))
     Vec<L> v[F1::E];
-    F1::template each<F1::RF>(it, [&](int e, int x, int) { v[e] = line_ld<NX>(line0, g, nl, x); });
+    F1::template each<F1::RF>(it, [&](int e, int x, int) { v[e] = line_ld<NX>((const C*)line0, g, nl, x); });
+    F1::template run<-1, true, false, false>(v, buf, ad1, twn, it);
+    const Real dk = prm<Real>(a.beta_dt, a.f.beta_dt);
+    F1::template each<F1::RL>(it, [&](int e, int k, int) {
+      // the odd factor is zero at the Nyquist index
+      const L kk = lbc<L>(2 * k == NX ? Real(0) : dk * Real(wrap_index(k, NX)));
+      v[e] = {lneg(lmul(kk, v[e].im)), lmul(kk, v[e].re)};
+    });
+    F1::template run<+1, true, true, true>(v, buf, ad1, twn, it);
+    fresh();
+    double s[CW];
+#pragma unroll
+    for (int q = 0; q < CW; ++q) s[q] = 0.0;
+    F1::template each<F1::RF>(it, [&](int e, int x, int) { lz_add(line_ld<NX>((const C*)line0, g, nl, x), v[e], s); });
+    double t = 0.0;
+#pragma unroll
+    for (int q = 0; q < CW; ++q) t -= (a.lo1 + a.h1 * ((l0 + CW * g + q) % a.ny)) * s[q];
+    t = block_sum(t, red);
+    if (tid == 0) a.part[bid] = t;
+  } else if constexpr (KIND == XP_FWD || KIND == XP_INV || KIND == XP_E) {
+    Vec<L> v[F1::E];
+    // X0 may read another field than the one it writes (aux)
+    const C* src = (KIND == XP_FWD && a.aux) ? reinterpret_cast<const C*>(a.aux) + (long long)l0 * NX : line0;
+    F1::template each<F1::RF>(it, [&](int e, int x, int) { v[e] = line_ld<NX>(src, g, nl, x); });
     F1::template run<(KIND == XP_FWD ? -1 : +1), true, false, false>(v, buf, ad1, twn, it);
     fresh();
     if constexpr (KIND == XP_E) __syncthreads();

@@ -81,11 +81,14 @@ __device__ __forceinline__ void head_tail(double k, double& h, double& t) {
 template <bool EXACT, typename L> struct TwoTerm { static constexpr bool v = false; };
 template <> struct TwoTerm<true, float2> { static constexpr bool v = true; };
 
-// x times an irrational constant, rounded once (EXACT float) or with the head alone
+// x times an irrational constant, rounded once (float: head and tail, in every
+// transform: sqrt(1/2) and sqrt(3)/2 are 1.7e-8 off as floats, and that gain
+// on half of the modes is what the dipolar energy, a small difference of large
+// ones, sees of a density transform's errors)
 template <bool EXACT, typename L> __device__ __forceinline__ L lkmul(L x, double k) {
   L h, t;
   head_tail(k, h, t);
-  if constexpr (TwoTerm<EXACT, L>::v) return lfma(x, h, lmul(x, t));
+  if constexpr (TwoTerm<true, L>::v) return lfma(x, h, lmul(x, t));
   else return lmul(x, h);
 }
 // a times the constant c + i DIR s

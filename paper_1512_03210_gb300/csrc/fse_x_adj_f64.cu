@@ -1,8 +1,9 @@
-// fse_x_adj_f64.cu -- x-pass instantiations for double: XP_R, XP_ADJ1, XP_ADJ2.
+// fse_x_adj_f64.cu -- x-pass instantiations for double: XP_R, XP_ADJ1, XP_ADJ2, XP_LZ.
 #include "fse_launch.cuh"
 
 namespace fse {
 template cudaError_t launch_xpass<double, XP_R>(int, const XArgs&, const void*, const void*, cudaStream_t);
 template cudaError_t launch_xpass<double, XP_ADJ1>(int, const XArgs&, const void*, const void*, cudaStream_t);
 template cudaError_t launch_xpass<double, XP_ADJ2>(int, const XArgs&, const void*, const void*, cudaStream_t);
+template cudaError_t launch_xpass<double, XP_LZ>(int, const XArgs&, const void*, const void*, cudaStream_t);
 }  // namespace fse
