@@ -163,6 +163,18 @@ fse_status fse_step_host(fse_plan_t plan, void* psi_host, double t0, int nsteps,
 fse_status fse_step_adjoint(fse_plan_t plan, const void* psi_n, void* g, double t_n,
                             const double* gamma_n, double* dgamma_n);
 
+/* Pull a cotangent back through nsteps consecutive steps from psi_0 (device,
+ * unchanged) at t0: the same as fse_step to each of the states and
+ * fse_step_adjoint from the last step to the first, with the kinetic half
+ * steps of neighbouring steps merged in both directions. states (device)
+ * is scratch for nsteps fields; g as in fse_step_adjoint; gamma_per_step (host,
+ * nullable) and dgamma (host, nullable) hold [nsteps][dim]. Synchronises the
+ * plan's stream. Errors: FSE_ERR_INVALID (null or misaligned buffers, nsteps <
+ * 1, precompute not run), FSE_ERR_UNSUPPORTED (as fse_step_adjoint). Uses the
+ * workspace's scratch wave function and spectrum. */
+fse_status fse_adjoint_sweep(fse_plan_t plan, const void* psi_0, void* states, void* g, double t0, int nsteps,
+                             const double* gamma_per_step, double* dgamma);
+
 /* Observables of psi (device, unchanged) at time t with trap frequencies
  * gamma (host, nullable, [dim]); float64 reductions on the device, one
  * device-to-host copy; synchronises the plan's stream. */

@@ -20,7 +20,7 @@ import numpy as np
 __all__ = [
     "load", "lib_path", "Plan", "FseParams", "FseObs", "FSE_OK", "FseError",
     "fse_plan_create", "fse_plan_set_workspace", "fse_kernel_precompute", "fse_step",
-    "fse_step_host", "fse_step_adjoint", "fse_observables", "fse_plan_set_stream",
+    "fse_step_host", "fse_step_adjoint", "fse_adjoint_sweep", "fse_observables", "fse_plan_set_stream",
     "fse_plan_destroy", "fse_status_string", "fse_plan_error", "fse_plan_launch_count",
     "header_functions", "to_params", "fse_plan_profile", "fse_plan_profile_read", "PASS_KINDS",
     "fse_mass_noalloc", "Batch", "fse_batch_create", "fse_batch_set_workspace", "fse_batch_precompute",
@@ -111,6 +111,7 @@ def load(build_if_missing: bool = True):
         "fse_step": (ct.c_int, [P, P, ct.c_double, ct.c_int, P]),
         "fse_step_host": (ct.c_int, [P, P, ct.c_double, ct.c_int, P]),
         "fse_step_adjoint": (ct.c_int, [P, P, P, ct.c_double, P, P]),
+        "fse_adjoint_sweep": (ct.c_int, [P, P, P, P, ct.c_double, ct.c_int, P, P]),
         "fse_observables": (ct.c_int, [P, P, ct.c_double, P, ct.POINTER(FseObs)]),
         "fse_plan_set_stream": (ct.c_int, [P, P]),
         "fse_plan_destroy": (ct.c_int, [P]),
@@ -242,6 +243,16 @@ def fse_step_adjoint(plan, psi_n, g, t_n: float, gamma_n=None, want_dgamma: bool
     _check(load().fse_step_adjoint(plan, _ptr(psi_n), _ptr(g), float(t_n), gp, dgp), "fse_step_adjoint", plan)
     del keep
     return dg if want_dgamma else None
+
+
+def fse_adjoint_sweep(plan, psi_0, states, g, t0: float, gammas, dim: int) -> np.ndarray:
+    """Pulls g back (in place) through len(gammas) steps from psi_0; returns dJ/dgamma [nsteps][dim]."""
+    keep, gp = _gammas(gammas)
+    dg = np.zeros((len(keep), dim), dtype=np.float64)
+    _check(load().fse_adjoint_sweep(plan, _ptr(psi_0), _ptr(states), _ptr(g), float(t0), len(keep), gp,
+                                    dg.ctypes.data_as(ct.c_void_p)), "fse_adjoint_sweep", plan)
+    del keep
+    return dg
 
 
 def fse_observables(plan, psi, t: float, gamma=None) -> FseObs:
@@ -443,6 +454,14 @@ class Plan:
 
     def adjoint(self, psi_n, g, t_n: float, gamma_n=None, want_dgamma=False):
         return fse_step_adjoint(self.handle, psi_n, g, t_n, gamma_n, want_dgamma, self.dim)
+
+    def adjoint_sweep(self, psi_0, g, t0: float, gammas):
+        """Pulls the cotangent g back (in place) through len(gammas) steps from psi_0; returns dJ/dgamma."""
+        import torch
+        assert psi_0.dtype == self.cdtype and psi_0.is_contiguous() and tuple(psi_0.shape) == self.shape
+        assert g.dtype == self.cdtype and g.is_contiguous() and tuple(g.shape) == self.shape
+        states = torch.empty((len(gammas),) + self.shape, dtype=self.cdtype, device=psi_0.device)
+        return fse_adjoint_sweep(self.handle, psi_0, states, g, t0, gammas, self.dim)
 
     def observables(self, psi, t: float, gamma=None) -> dict:
         return fse_observables(self.handle, psi, t, gamma).as_dict(self.dim)

@@ -4,8 +4,8 @@
 steps with per-step trap frequencies ``gammas`` ([nsteps][dim], float64) and
 is differentiable with respect to both. The forward pass keeps one state
 every ceil(sqrt(T)) steps; the backward pass recomputes the states of each
-segment with ``fse_step`` and pulls the cotangent back with
-``fse_step_adjoint``, last step first. Gradients follow torch's convention for
+segment and pulls the cotangent back through it, last step first, with
+``fse_adjoint_sweep``. Gradients follow torch's convention for
 complex inputs, dJ/dRe + i dJ/dIm, which is the library's cotangent
 convention.
 """
@@ -45,13 +45,7 @@ class _Evolve(torch.autograd.Function):
         for si in range(len(ctx.ckpts) - 1, -1, -1):
             s0 = si * seg
             n = min(seg, T - s0)
-            states = [ctx.ckpts[si]]
-            x = ctx.ckpts[si].clone()
-            for k in range(n - 1):
-                plan.step(x, t0 + (s0 + k) * dt, 1, gam[s0 + k:s0 + k + 1])
-                states.append(x.clone())
-            for k in range(n - 1, -1, -1):
-                dgam[s0 + k] = plan.adjoint(states[k], g, t0 + (s0 + k) * dt, gam[s0 + k], want_dgamma=True)[:plan.dim]
+            dgam[s0:s0 + n] = plan.adjoint_sweep(ctx.ckpts[si], g, t0 + s0 * dt, gam[s0:s0 + n])
         ctx.ckpts = None
         return g, torch.as_tensor(dgam, dtype=ctx.gdtype, device=ctx.gdev), None, None
 

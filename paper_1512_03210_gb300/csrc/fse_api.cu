@@ -319,7 +319,7 @@ void lattice_nodes(fse_plan* P, double ta, double tb, XArgs& a) {
 // (3D) or fwd-y . phase . inv-y (2D). On exit the field is x-spectral.
 // f selects the plan's kinetic table: 1 the half step (dt/2; w1 dt/2 at order
 // 4), 2 two merged half steps (dt; w1 dt), 3 the middle of the fourth-order
-// composition ((w1 + w0) dt / 2); -1 the conjugate half step (adjoint).
+// composition ((w1 + w0) dt / 2); -1 and -2 the conjugates of 1 and 2 (adjoint).
 fse_status kinetic_yz(fse_plan* P, void* psi, double f, double dt) {
   (void)dt;  // the phase tables were built with the plan's dt
   MulArgs m;
@@ -327,12 +327,12 @@ fse_status kinetic_yz(fse_plan* P, void* psi, double f, double dt) {
   m.mode = MUL_KIN;
   if (f == 1.0 || f == -1.0) {
     m.kin = P->ws_ptr(P->off_kin_half);
-  } else if (f == 2.0) {
+  } else if (f == 2.0 || f == -2.0) {
     m.kin = P->ws_ptr(P->off_kin_full);
   } else if (f == 3.0 && P->p.order == 4) {
     m.kin = P->ws_ptr(P->off_kin_mid);
   } else {
-    return fail(P, FSE_ERR_INVALID, "kinetic table selector must be 1, 2, 3 (order 4) or -1");
+    return fail(P, FSE_ERR_INVALID, "kinetic table selector must be 1, 2, 3 (order 4), -1 or -2");
   }
   m.conj = f < 0.0;
   m.lx = P->nx;

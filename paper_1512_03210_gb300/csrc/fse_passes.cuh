@@ -36,7 +36,7 @@ struct XArgs {
   double lo0, lo1, lo2, h0, h1, h2;
   double* part;           // pass R: partial of sum varphi |psi|^2; passes E / XI: partial of sum |u1|^2
   const double* scale;    // pass A: optional renormalisation factor (device scalar)
-  const void* aux;        // adjoint passes: u1 (output of the first kinetic half step)
+  const void* aux;        // adjoint passes, A: u1 (output of the first kinetic half step); X0: its input
   long long part_stride;  // adjoint pass 1: distance between the three gradient slots
   double dp[12];          // adjoint pass 1: dP/dgamma_v = dp[4v] x^2 + dp[4v+1] y^2 + dp[4v+2] x y + dp[4v+3] z^2
   // optical lattice lat_amp sum_v sin^2(lat_k[v] x_v): its integral over the
@@ -46,7 +46,7 @@ struct XArgs {
   double lat_k[3];
   int lat_nq;
   double lat_w[16], lat_c[16], lat_s[16];
-  void* out;              // pass R: optional real array receiving varphi (the nonlocal potential)
+  void* out;              // pass R: optional real array receiving varphi (the nonlocal potential); E, XI: u1
   // float copies of the scalars above (see MulArgs::f)
   struct {
     float beta_dt, lam, pa, pb, pc, pe, lo0, lo1, lo2, h0, h1, h2;
@@ -565,14 +565,15 @@ __device__ __forceinline__ void xpass_body(const XArgs& a, const typename TwOf<R
     if (tid == 0) a.part[bid] = t;
   } else if constexpr (KIND == XP_FWD || KIND == XP_INV || KIND == XP_E) {
     Vec<L> v[F1::E];
-    // X0 may read another field than the one it writes (aux)
+    // X0 may read another field than the one it writes (aux), E and XI may write another (out)
     const C* src = (KIND == XP_FWD && a.aux) ? reinterpret_cast<const C*>(a.aux) + (long long)l0 * NX : line0;
     F1::template each<F1::RF>(it, [&](int e, int x, int) { v[e] = line_ld<NX>(src, g, nl, x); });
     F1::template run<(KIND == XP_FWD ? -1 : +1), true, false, false>(v, buf, ad1, twn, it);
     fresh();
     if constexpr (KIND == XP_E) __syncthreads();
+    C* dst = (KIND != XP_FWD && a.out) ? reinterpret_cast<C*>(a.out) + (long long)l0 * NX : line0;
     F1::template each<F1::RL>(it, [&](int e, int x, int) {
-      line_st<NX>(line0, g, nl, x, v[e]);
+      line_st<NX>(dst, g, nl, x, v[e]);
       if constexpr (KIND == XP_E) real_st<RS>(field, g, x, lfma(v[e].re, v[e].re, lmul(v[e].im, v[e].im)));
     });
     if constexpr (KIND != XP_FWD) {
@@ -598,7 +599,7 @@ __device__ __forceinline__ void xpass_body(const XArgs& a, const typename TwOf<R
       // the tile's rows of psi (contiguous) move to L2 while the C2R runs (the
       // bulk prefetch needs a 16-byte aligned start; psi may be only
       // element-aligned, and every line then starts 16-byte aligned too)
-      prefetch_l2_bulk(line0, (unsigned)(min(LN, nl) * NX * sizeof(C)));
+      if (!a.aux) prefetch_l2_bulk(line0, (unsigned)(min(LN, nl) * NX * sizeof(C)));
     }
     if (a.use_spec) c2r();
     fresh();
@@ -705,8 +706,10 @@ __device__ __forceinline__ void xpass_body(const XArgs& a, const typename TwOf<R
         // thread: a conversion from double issues on the narrow FP64 pipe.
         const bool rescale = a.scale != nullptr;
         const L fsc = lbc<L>(rescale ? Real(*a.scale) : Real(1));
+        // u1 lies in psi, or in another field (aux)
+        const C* u1 = a.aux ? reinterpret_cast<const C*>(a.aux) + (long long)l0 * NX : (const C*)line0;
         Vec<L> v[F1::E];
-        F1::template each<F1::RF>(it, [&](int e, int x, int) { v[e] = line_ld<NX>((const C*)line0, g, nl, x); });
+        F1::template each<F1::RF>(it, [&](int e, int x, int) { v[e] = line_ld<NX>(u1, g, nl, x); });
         F1::template each<F1::RF>(it, [&](int e, int x, int) {
           const Vec<L> u = v[e];
           const L rho = lfma(u.re, u.re, lmul(u.im, u.im));
