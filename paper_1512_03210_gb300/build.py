@@ -17,9 +17,11 @@ PEAKS_LIB = os.path.join(OUT, "libfse_peaks.so")
 INCLUDE = os.path.join(ROOT, "include")
 
 SOURCES = ["fse_api.cu", "fse_precompute.cu", "fse_observables.cu", "fse_adjoint.cu",
-           "fse_col_plain_f32.cu", "fse_col_kin_f32.cu", "fse_col_pad_f32.cu", "fse_col_khat_f32.cu",
+           "fse_col_plain_f32.cu", "fse_col_deriv_f32.cu", "fse_col_kin_f32.cu", "fse_col_pad_f32.cu",
+           "fse_col_khat_f32.cu", "fse_col_khat2_f32.cu",
            "fse_col_plain_f64.cu", "fse_col_kin_f64.cu", "fse_col_pad_f64.cu", "fse_col_khat_f64.cu",
-           "fse_x_e_f32.cu", "fse_x_a_f32.cu", "fse_x_adj_f32.cu", "fse_x_e_f64.cu", "fse_x_a_f64.cu",
+           "fse_x_e_f32.cu", "fse_x_a_f32.cu", "fse_x_adj_f32.cu", "fse_x_real_f32.cu",
+           "fse_x_e_f64.cu", "fse_x_a_f64.cu",
            "fse_x_adj_f64.cu", "fse_noalloc.cu", "fse_batch.cu", "fse_batch_col.cu", "fse_batch_x.cu",
            "fse_ground.cu", "fse_gs_f32.cu", "fse_gs_f64.cu"]
 HEADERS = ["fse_fft.cuh", "fse_vec.cuh", "fse_col.cuh", "fse_passes.cuh", "fse_launch.cuh", "fse_gsx.cuh", "fse_batch.cuh", "fse_internal.h"]

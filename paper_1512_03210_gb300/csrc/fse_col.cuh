@@ -504,7 +504,7 @@ template <typename Real, int N, int VAR, int NP, bool PDL>
 __device__ __forceinline__ void col_body(const ColArgs& a, const MulArgs& m, const typename TwOf<Real>::T* __restrict__ tw,
                                          int bid) {
   typedef ColCfg<Real, N, VAR, NP> K;
-  if constexpr (K::S::TWO) {
+  if constexpr (K::S::TWO && VAR != COL_KHAT2) {  // (a 2D pass is one plane: nothing to gather)
     const int ngat = a.tail > 0 ? (a.nplanes * a.tail + K::NC - 1) / K::NC : 0;
     if (bid < ngat) col_tile<Real, N, VAR, NP, true, PDL>(a, m, tw, bid, ngat);
     else col_tile<Real, N, VAR, NP, false, PDL>(a, m, tw, bid, ngat);
