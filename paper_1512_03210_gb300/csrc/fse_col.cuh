@@ -148,7 +148,7 @@ struct ColCfg {
   // float64 passes with eight elements, 96 up to 12 elements, 80 or 64 below
   __host__ __device__ static constexpr int minb() {
     const int thr = E > 12 || (sizeof(Real) == 8 && E > 6) ? 512
-                                                           : (E > 8 || sizeof(Real) == 8 ? 640 : (S::KHAT ? 768 : 1024));
+                                                           : (E > 8 || sizeof(Real) == 8 || VAR == COL_LZ ? 640 : (S::KHAT ? 768 : 1024));
     const int b = thr / ((NT + 31) / 32 * 32);
     return b < 1 ? 1 : (b > 32 ? 32 : b);
   }
@@ -225,13 +225,19 @@ __device__ __forceinline__ double lane_of(const double (&v)[1]) { return v[0]; }
 __device__ __forceinline__ float2 lane_ld(const float* p) { return *reinterpret_cast<const float2*>(p); }
 __device__ __forceinline__ double lane_ld(const double* p) { return *p; }
 
-// s += Im(conj(u) d) per lane, in float64
-__device__ __forceinline__ void lz_add(const Vec<float2>& u, const Vec<float2>& d, double (&s)[2]) {
-  s[0] += (double)u.re.x * d.im.x - (double)u.im.x * d.re.x;
-  s[1] += (double)u.re.y * d.im.y - (double)u.im.y * d.re.y;
+// s += Im(conj(u) d), u scaled by su and d by sd
+template <typename L>
+__device__ __forceinline__ void lz_add(const Vec<L>& u, const Vec<L>& d, const L& su, const L& sd, ExactSum<L>& s) {
+  const L re = lmul(su, u.re), im = lneg(lmul(su, u.im));
+  s.prod(re, lmul(sd, d.im));
+  s.prod(im, lmul(sd, d.re));
 }
-__device__ __forceinline__ void lz_add(const Vec<double>& u, const Vec<double>& d, double (&s)[1]) {
-  s[0] += u.re * d.im - u.im * d.re;
+// max modulus of the components of the elements a thread holds before (after)
+// the transforms; a length that leaves threads short of items leaves elements unset
+template <typename F, typename L, int E> __device__ __forceinline__ float vmax_abs(int it, const Vec<L> (&v)[E]) {
+  float m = 0.f;
+  F::template each<F::RF>(it, [&](int e, int, int) { m = lmax_abs(lmax_abs(m, v[e].re), v[e].im); });
+  return m;
 }
 
 template <typename Real, int N, int VAR, int NP, bool GATHER, bool PDL>
@@ -386,6 +392,8 @@ __device__ __forceinline__ void col_tile(const ColArgs& a, const MulArgs& m, con
     F::template each<RF>(it, [&](int e, int row, int) { col_st(geo, row * ls, v[e]); });
   } else if constexpr (VAR == COL_DY || VAR == COL_LZ) {
     F::template each<RF>(it, [&](int e, int row, int) { v[e] = col_ld(geo, row * ls); });
+    float um = 0.f;
+    if constexpr (VAR == COL_LZ) um = vmax_abs<F>(it, v);
     F::template run<-1, true, false, false>(v, buf, addr, tw, it);
     const Real dk = prm<Real>(m.dkr, m.f.dkr);  // includes 1/N
     F::template each<RL>(it, [&](int e, int row, int) {
@@ -397,14 +405,15 @@ __device__ __forceinline__ void col_tile(const ColArgs& a, const MulArgs& m, con
     fresh();
     if constexpr (VAR == COL_LZ) {
       __shared__ double red[32];
-      double s[CW];
-#pragma unroll
-      for (int q = 0; q < CW; ++q) s[q] = 0.0;
-      F::template each<RF>(it, [&](int e, int row, int) { lz_add(col_ld(geo, row * ls), v[e], s); });
+      // (the thread's rows here are the ones it loaded at first)
+      const Pow2<L> su = pow2_scale<L>(um), sd = pow2_scale<L>(vmax_abs<F>(it, v));
+      ExactSum<L> s;
+      F::template each<RF>(it, [&](int e, int row, int) { lz_add(col_ld(geo, row * ls), v[e], su.scale, sd.scale, s); });
       double t = 0.0;
 #pragma unroll
       for (int q = 0; q < CW; ++q)
-        if (geo.ok[q]) t += (a.lo + a.h * geo.px[q]) * s[q];
+        if (geo.ok[q]) t += (a.lo + a.h * geo.px[q]) * s.get(q);
+      t *= su.inv * sd.inv;
       t = block_sum(t, red);
       if (tid == 0) a.part[bid] = t;
       return;

@@ -35,41 +35,111 @@ struct ObsArgs {
   double lat_amp, lat_k[3];  // optical lattice lat_amp sum_v sin^2(lat_k[v] x_v)
 };
 
-// Moments of the density in float64, one warp per line, in index units from
-// the grid's middle (exact): along a line only the sums of rho, rho^2, rho i
-// and rho i^2 are formed, and a line's y and z enter once; the coordinates and
-// the harmonic trap energy follow from the sums on the host. About 13 float64
-// slots per point in place of 45 (128^3: 172 -> 50 us, the FP64 pipe's time).
-// Slots: rho, rho^2, lattice energy, and rho times i, j, k, i i, j j, k k, i j.
+// CW points of a line 32 apart (zero past the end)
 template <typename Real>
-__global__ void __launch_bounds__(256) k_obs_phys(const typename Cplx<Real>::T* __restrict__ psi, ObsArgs o, int nz,
+__device__ __forceinline__ Vec<typename LaneOf<Real>::T> pair_at(const typename Cplx<Real>::T* row, int x, int nx) {
+  constexpr int CW = sizeof(typename LaneOf<Real>::T) / sizeof(Real);
+  Real re[CW], im[CW];
+#pragma unroll
+  for (int q = 0; q < CW; ++q) {
+    const bool in = x + 32 * q < nx;
+    re[q] = in ? row[x + 32 * q].x : Real(0);
+    im[q] = in ? row[x + 32 * q].y : Real(0);
+  }
+  return {lane_of(re), lane_of(im)};
+}
+
+// lattice energy of a lane's points of a line
+template <typename C> __device__ __forceinline__ double lattice_line(const C* row, const ObsArgs& o, int iy, int iz, int lane) {
+  const double y = o.lo[1] + o.h[1] * iy, z = o.lo[2] + o.h[2] * iz;
+  double acc = 0.0;
+  for (int x = lane; x < o.nx; x += 32) {
+    const C u = row[x];
+    const double rho = (double)u.x * u.x + (double)u.y * u.y, xx = o.lo[0] + o.h[0] * x;
+    const double sx = sin(o.lat_k[0] * (o.c * xx + o.s * y)), sy = sin(o.lat_k[1] * (-o.s * xx + o.c * y)),
+                 sz = sin(o.lat_k[2] * z);
+    acc += o.lat_amp * (sx * sx + sy * sy + sz * sz) * rho;
+  }
+  return acc;
+}
+
+// Moments of the density, one warp per line, in index units from the grid's
+// middle (exact): along a line only the sums of rho, rho^2, rho i and rho i^2
+// are formed, and a line's y and z enter once; the coordinates and the harmonic
+// trap energy follow from the sums on the host. In float64 that is about 11
+// slots of the FP64 pipe per point in place of 45 (128^3 float32 fields: 172 ->
+// 56 us, the pipe's time); float fields are summed by three floats (ExactSum):
+// 33 us, the chains of two-sums of the 16 warps that 126 registers leave an SM.
+// Slots: rho, rho^2, lattice energy, and rho times i, j, k, i i, j j, k k, i j.
+__global__ void __launch_bounds__(256) k_obs_phys(const float2* __restrict__ psi, ObsArgs o, int nz, double* part) {
+  __shared__ double red[10 * 256];
+  typedef ExactSum<float2> Sum;
+  const int lane = threadIdx.x & 31, nw = gridDim.x * 8;
+  Sum t0, t1, ti, tj, tk, tii, tjj, tkk, tij;
+  double lat = 0.0;
+  RunScale<float2> su;
+  for (int l = blockIdx.x * 8 + (threadIdx.x >> 5); l < o.nlines; l += nw) {
+    const float2* row = psi + (long long)l * o.nx;
+    const int iy = l % o.ny, iz = l / o.ny;
+    float um = 0.f;
+#pragma unroll 2
+    for (int x = lane; x < o.nx; x += 64) {
+      const Vec<float2> u = pair_at<float>(row, x, o.nx);
+      um = lmax_abs(lmax_abs(um, u.re), u.im);
+    }
+    su.grow(um, [&](float2 r) {
+      const float2 r2 = lmul(r, r);
+      t0.rescale(r2), ti.rescale(r2), tj.rescale(r2), tk.rescale(r2), tii.rescale(r2), tjj.rescale(r2);
+      tkk.rescale(r2), tij.rescale(r2), t1.rescale(lmul(r2, r2));
+    });
+    Sum s0, s1;
+#pragma unroll 2
+    for (int x = lane; x < o.nx; x += 64) {
+      const Vec<float2> u = pair_at<float>(row, x, o.nx);
+      const Sum rho = Sum::density(lmul(su.scale, u.re), lmul(su.scale, u.im));
+      const float i = (float)(x - o.nx / 2);
+      const float2 i2 = make_float2(i, i + 32.f);
+      s0.add(rho);
+      s1.prod(i2, rho);
+      tii.prod(lmul(i2, i2), rho);
+      t1.square(rho);
+    }
+    if (o.lat_amp != 0.0) lat += lattice_line(row, o, iy, iz, lane);
+    const float j = (float)(iy - o.ny / 2), k = (float)(iz - nz / 2);
+    const float2 j2 = make_float2(j, j), k2 = make_float2(k, k);
+    t0.add(s0);
+    ti.add(s1);
+    tj.prod(j2, s0);
+    tk.prod(k2, s0);
+    tjj.prod(lmul(j2, j2), s0);
+    tkk.prod(lmul(k2, k2), s0);
+    tij.prod(j2, s1);
+  }
+  const double v2 = su.inv * su.inv;
+  auto val = [&](const Sum& s) { return v2 * (s.get(0) + s.get(1)); };
+  const double acc[10] = {val(t0), v2 * val(t1), lat, val(ti), val(tj), val(tk), val(tii), val(tjj), val(tkk), val(tij)};
+  block_sums(acc, red, [&](int k, double v) { part[k * kPartStride + blockIdx.x] = v; });
+}
+
+__global__ void __launch_bounds__(256) k_obs_phys(const double2* __restrict__ psi, ObsArgs o, int nz,
                                                   double* part) {
   __shared__ double red[10 * 256];
   const int lane = threadIdx.x & 31, nw = gridDim.x * 8;
   double acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   for (int l = blockIdx.x * 8 + (threadIdx.x >> 5); l < o.nlines; l += nw) {
-    const typename Cplx<Real>::T* row = psi + (long long)l * o.nx;
+    const double2* row = psi + (long long)l * o.nx;
     const int iy = l % o.ny, iz = l / o.ny;
     double s0 = 0.0, s1 = 0.0, i0 = lane - o.nx / 2;
 #pragma unroll 4
     for (int x = lane; x < o.nx; x += 32, i0 += 32.0) {
-      const typename Cplx<Real>::T u = row[x];
-      const double rho = (double)u.x * u.x + (double)u.y * u.y, t = rho * i0;
+      const double2 u = row[x];
+      const double rho = u.x * u.x + u.y * u.y, t = rho * i0;
       s0 += rho;
       acc[1] = fma(rho, rho, acc[1]);
       s1 += t;
       acc[6] = fma(t, i0, acc[6]);
     }
-    if (o.lat_amp != 0.0) {
-      const double y = o.lo[1] + o.h[1] * iy, z = o.lo[2] + o.h[2] * iz;
-      for (int x = lane; x < o.nx; x += 32) {
-        const typename Cplx<Real>::T u = row[x];
-        const double rho = (double)u.x * u.x + (double)u.y * u.y, xx = o.lo[0] + o.h[0] * x;
-        const double sx = sin(o.lat_k[0] * (o.c * xx + o.s * y)), sy = sin(o.lat_k[1] * (-o.s * xx + o.c * y)),
-                     sz = sin(o.lat_k[2] * z);
-        acc[2] += o.lat_amp * (sx * sx + sy * sy + sz * sz) * rho;
-      }
-    }
+    if (o.lat_amp != 0.0) acc[2] += lattice_line(row, o, iy, iz, lane);
     const double j = iy - o.ny / 2, k = iz - nz / 2, a = j * s0, b = k * s0;
     acc[0] += s0;
     acc[3] += s1;
@@ -89,19 +159,43 @@ __global__ void __launch_bounds__(256) k_obs_kin(const typename Cplx<Real>::T* _
                                                  double* part) {
   __shared__ double red[32];
   const int lane = threadIdx.x & 31, nw = gridDim.x * 8;
-  double acc = 0.0;
+  typedef typename LaneOf<Real>::T L;
+  constexpr int CW = sizeof(L) / sizeof(Real);
+  ExactSum<L> sum;
+  RunScale<L> su;
+  // the weights grow with |k|: their scale is the corner's
+  const Real cx = Real(dkx) * Real(o.nx / 2), cy = Real(dky) * Real(o.ny / 2), cz = Real(dkz) * Real(nz / 2);
+  const Pow2<L> sw = pow2_scale<L>((float)pow(cx * cx + cy * cy + cz * cz + Real(m2), Real(s)));
   for (int l = blockIdx.x * 8 + (threadIdx.x >> 5); l < o.nlines; l += nw) {
     const typename Cplx<Real>::T* row = sp + (long long)l * o.nx;
     const Real ky = Real(dky) * Real(wrap_index(l % o.ny, o.ny));
     const Real kz = nz > 1 ? Real(dkz) * Real(wrap_index(l / o.ny, nz)) : Real(0);
-#pragma unroll 4
-    for (int x = lane; x < o.nx; x += 32) {
-      const Real kx = Real(dkx) * Real(wrap_index(x, o.nx));
-      const Real k2 = kx * kx + ky * ky + kz * kz + Real(m2);
-      const typename Cplx<Real>::T u = row[x];
-      acc += (double)pow(k2, Real(s)) * ((double)u.x * u.x + (double)u.y * u.y);
+    auto at = [&](int x) { return pair_at<Real>(row, x, o.nx); };
+    float um = 0.f;
+    if constexpr (sizeof(Real) == 4) {
+#pragma unroll 2
+      for (int x = lane; x < o.nx; x += 64) {
+        const Vec<L> u = at(x);
+        um = lmax_abs(lmax_abs(um, u.re), u.im);
+      }
+    }
+    su.grow(um, [&](L r) { sum.rescale(lmul(r, r)); });
+#pragma unroll 2
+    for (int x = lane; x < o.nx; x += 32 * CW) {
+      Real w[CW];
+#pragma unroll
+      for (int q = 0; q < CW; ++q) {
+        const Real kx = Real(dkx) * Real(wrap_index(x + 32 * q, o.nx));
+        w[q] = x + 32 * q < o.nx ? pow(kx * kx + ky * ky + kz * kz + Real(m2), Real(s)) : Real(0);
+      }
+      const Vec<L> u = at(x);
+      sum.dens(lmul(sw.scale, lane_of(w)), lmul(su.scale, u.re), lmul(su.scale, u.im));
     }
   }
+  double acc = 0.0;
+#pragma unroll
+  for (int q = 0; q < CW; ++q) acc += sum.get(q);
+  acc *= sw.inv * (su.inv * su.inv);
   const double v = block_sum(acc, red);
   if (threadIdx.x == 0) part[SL_KIN * kPartStride + blockIdx.x] = v;
 }
@@ -268,7 +362,7 @@ fse_status observables(fse_plan* P, const void* psi_in, double t, const double* 
   }
 
   cudaEvent_t ev = prof_begin(P);
-  k_obs_phys<Real><<<blocks, 256, 0, P->stream>>>(psi, o, P->nz, part);
+  k_obs_phys<<<blocks, 256, 0, P->stream>>>(psi, o, P->nz, part);
   prof_end(P, FSE_PASS_OTHER, ev);
   if ((st = launched(P, cudaGetLastError(), "observables")) != FSE_OK) return st;
   for (int k = SL_MASS; k <= SL_XY; ++k) cnt.n[k] = blocks;

@@ -545,6 +545,7 @@ __device__ __forceinline__ void xpass_body(const XArgs& a, const typename TwOf<R
     // partial of -sum y Im(conj(psi) d_x psi), d_x by the line's own transforms (beta_dt: 2 pi / (W n))
     Vec<L> v[F1::E];
     F1::template each<F1::RF>(it, [&](int e, int x, int) { v[e] = line_ld<NX>((const C*)line0, g, nl, x); });
+    const float um = vmax_abs<F1>(it, v);
     F1::template run<-1, true, false, false>(v, buf, ad1, twn, it);
     const Real dk = prm<Real>(a.beta_dt, a.f.beta_dt);
     F1::template each<F1::RL>(it, [&](int e, int k, int) {
@@ -554,13 +555,15 @@ __device__ __forceinline__ void xpass_body(const XArgs& a, const typename TwOf<R
     });
     F1::template run<+1, true, true, true>(v, buf, ad1, twn, it);
     fresh();
-    double s[CW];
-#pragma unroll
-    for (int q = 0; q < CW; ++q) s[q] = 0.0;
-    F1::template each<F1::RF>(it, [&](int e, int x, int) { lz_add(line_ld<NX>((const C*)line0, g, nl, x), v[e], s); });
+    const Pow2<L> su = pow2_scale<L>(um), sd = pow2_scale<L>(vmax_abs<F1>(it, v));
+    ExactSum<L> s;
+    F1::template each<F1::RF>(it, [&](int e, int x, int) {
+      lz_add(line_ld<NX>((const C*)line0, g, nl, x), v[e], su.scale, sd.scale, s);
+    });
     double t = 0.0;
 #pragma unroll
-    for (int q = 0; q < CW; ++q) t -= (a.lo1 + a.h1 * ((l0 + CW * g + q) % a.ny)) * s[q];
+    for (int q = 0; q < CW; ++q) t -= (a.lo1 + a.h1 * ((l0 + CW * g + q) % a.ny)) * s.get(q);
+    t *= su.inv * sd.inv;
     t = block_sum(t, red);
     if (tid == 0) a.part[bid] = t;
   } else if constexpr (KIND == XP_FWD || KIND == XP_INV || KIND == XP_E) {
@@ -612,24 +615,31 @@ __device__ __forceinline__ void xpass_body(const XArgs& a, const typename TwOf<R
       // varphi itself, as a real field in the layout of psi, and (or) the sum
       // over the tile of varphi |psi|^2 (nonlocal interaction energy density)
       Real* phi = reinterpret_cast<Real*>(a.out);
-      double acc = 0.0;
-      F1::template each<F1::RF>(it, [&](int, int x, int) {
-        const L p = phi_at(x);
-        if (phi) {
+      if (phi) {
+        F1::template each<F1::RF>(it, [&](int, int x, int) {
+          const L p = phi_at(x);
 #pragma unroll
           for (int q = 0; q < CW; ++q)
             if (CW * g + q < nl) phi[(long long)(l0 + CW * g + q) * NX + x] = lane_get(p, q);
-        }
-        if (a.part) {
-#pragma unroll
-          for (int q = 0; q < CW; ++q)
-            if (CW * g + q < nl) {
-              const C u = line0[(CW * g + q) * NX + x];
-              acc += (double)lane_get(p, q) * ((double)u.x * u.x + (double)u.y * u.y);
-            }
-        }
-      });
+        });
+      }
       if (!a.part) return;
+      float pm = 0.f;
+      Vec<L> u[F1::E];
+      F1::template each<F1::RF>(it, [&](int e, int x, int) {
+        u[e] = line_ld<NX>((const C*)line0, g, nl, x);
+        pm = lmax_abs(pm, phi_at(x));
+      });
+      const Pow2<L> su = pow2_scale<L>(vmax_abs<F1>(it, u)), sp = pow2_scale<L>(pm);
+      ExactSum<L> sum;
+      F1::template each<F1::RF>(it, [&](int e, int x, int) {
+        sum.dens(lmul(sp.scale, phi_at(x)), lmul(su.scale, u[e].re), lmul(su.scale, u[e].im));
+      });
+      double acc = 0.0;
+#pragma unroll
+      for (int q = 0; q < CW; ++q)
+        if (CW * g + q < nl) acc += sum.get(q);
+      acc *= sp.inv * (su.inv * su.inv);
       acc = block_sum(acc, red);
       if (tid == 0) a.part[bid] = acc;
     } else if constexpr (KIND == XP_ADJ2) {
@@ -662,20 +672,28 @@ __device__ __forceinline__ void xpass_body(const XArgs& a, const typename TwOf<R
           line_st<NX>(line0, g, nl, x, phase_mul(gu, lneg(th)));
         });
         if (a.part) {
-          // sums over the thread's part of its lines of r, r X and r X^2 in float64
+          // sums over the thread's part of its lines of r, r X and r X^2, by
+          // those of r, r i and r i^2 with i the index from the middle
+          float rm = 0.f;
+          F1::template each<F1::RF>(it, [&](int e, int, int) { rm = lmax_abs(rm, rr[e]); });
+          const Pow2<L> sr = pow2_scale<L>(rm);
+          ExactSum<L> e0, e1, e2;
+          F1::template each<F1::RF>(it, [&](int e, int x, int) {
+            const L r = lmul(sr.scale, rr[e]);
+            const Real i = Real(x - NX / 2);
+            e0.add(r);
+            e1.prod(r, lane_bc<L>(i));
+            e2.prod(r, lane_bc<L>(i * i));
+          });
+          const double xc = a.lo0 + a.h0 * (NX / 2);
           double s0[CW], s1[CW], s2[CW];
 #pragma unroll
-          for (int q = 0; q < CW; ++q) s0[q] = s1[q] = s2[q] = 0.0;
-          F1::template each<F1::RF>(it, [&](int e, int x, int) {
-            const double X = a.lo0 + a.h0 * x;
-#pragma unroll
-            for (int q = 0; q < CW; ++q) {
-              const double rd = (double)lane_get(rr[e], q), rx = rd * X;
-              s0[q] += rd;
-              s1[q] += rx;
-              s2[q] = fma(rx, X, s2[q]);
-            }
-          });
+          for (int q = 0; q < CW; ++q) {
+            const double i1 = a.h0 * (sr.inv * e1.get(q)), i2 = a.h0 * a.h0 * (sr.inv * e2.get(q));
+            s0[q] = sr.inv * e0.get(q);
+            s1[q] = fma(xc, s0[q], i1);
+            s2[q] = fma(xc, s1[q] + i1, i2);
+          }
           // dP/dgamma_v = dp[4v] X^2 + dp[4v+1] Y^2 + dp[4v+2] X Y + dp[4v+3] Z^2
           double dg[3] = {0.0, 0.0, 0.0};
 #pragma unroll

