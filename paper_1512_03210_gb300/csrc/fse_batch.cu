@@ -37,7 +37,7 @@ struct fse_batch {
     int nx = 0, ny = 0;
     std::vector<int> runs;
     fse_plan* plan = nullptr;  // twiddles and kernel transform of the group (shared by its runs)
-    size_t off_plan = 0, off_desc = 0;
+    size_t off_plan = 0, off_desc = 0, off_trap = 0;
   };
   std::vector<fse_params> runs;
   std::vector<Group> groups;
@@ -135,6 +135,8 @@ fse_status fse_batch_create(const fse_params* runs, int nruns, void* stream, fse
     off = al(off + nb);
     G.off_desc = off;
     off = al(off + sizeof(BatchRun) * G.runs.size());
+    G.off_trap = off;
+    off = al(off + sizeof(float4) * kTrapSteps * G.runs.size());
     const size_t kin_bytes = (size_t)(G.nx / 2 + 1) * (G.ny / 2 + 1) * 8;
     const size_t spec_bytes = (size_t)G.ny * G.plan->sx * 8;
     for (size_t k = 1; k < G.runs.size(); ++k) {
@@ -212,6 +214,7 @@ fse_status batch_sequence(fse_batch* B, int nsteps, cudaStream_t st0, long long*
     fse_plan* P = G.plan;
     const int nr = (int)G.runs.size();
     const BatchRun* ddesc = reinterpret_cast<const BatchRun*>(B->ptr(G.off_desc));
+    float4* trap = reinterpret_cast<float4*>(B->ptr(G.off_trap));
     const bool nl_on = B->runs[G.runs[0]].kernel != FSE_KERNEL_NONE;
     XArgs xa = x_args(P, nullptr, nl_on ? reinterpret_cast<void*>(1) : nullptr);  // pointers come from the table
     xa.use_spec = nl_on ? 1 : 0;
@@ -241,22 +244,25 @@ fse_status batch_sequence(fse_batch* B, int nsteps, cudaStream_t st0, long long*
       return FSE_OK;
     };
     fse_status s;
-    if ((s = chk(launch_xb(XP_FWD, P->nx, xa, twn, tw2n, ddesc, nr, t0, 0, st), "batch x")) != FSE_OK) return s;
+    if ((s = chk(launch_xb(XP_FWD, P->nx, xa, twn, tw2n, ddesc, nr, trap, st), "batch x")) != FSE_OK) return s;
     for (int n = 0; n < nsteps; ++n) {
+      if (n % kTrapSteps == 0 &&
+          (s = chk(launch_batch_trap(ddesc, nr, t0, n, std::min(kTrapSteps, nsteps - n), trap, st), "batch trap")) != FSE_OK)
+        return s;
       if ((s = chk(launch_colb<COL_KIN2>(P->ny, ck, mk1, twy, ddesc, nr, n > 0, st), "batch kinetic")) != FSE_OK)
         return s;
       if (nl_on) {
-        if ((s = chk(launch_xb(XP_E, P->nx, xa, twn, tw2n, ddesc, nr, t0, n, st), "batch density")) != FSE_OK) return s;
+        if ((s = chk(launch_xb(XP_E, P->nx, xa, twn, tw2n, ddesc, nr, trap, st), "batch density")) != FSE_OK) return s;
         if ((s = chk(launch_colb<COL_KHAT2>(P->ny, cg, mk2, tw2y, ddesc, nr, 0, st), "batch kernel")) != FSE_OK)
           return s;
       } else {
-        if ((s = chk(launch_xb(XP_INV, P->nx, xa, twn, tw2n, ddesc, nr, t0, n, st), "batch x")) != FSE_OK) return s;
+        if ((s = chk(launch_xb(XP_INV, P->nx, xa, twn, tw2n, ddesc, nr, trap, st), "batch x")) != FSE_OK) return s;
       }
-      if ((s = chk(launch_xb(XP_A, P->nx, xa, twn, tw2n, ddesc, nr, t0, n, st), "batch phase")) != FSE_OK) return s;
+      if ((s = chk(launch_xb(XP_A, P->nx, xa, twn, tw2n, ddesc, nr, trap + (size_t)(n % kTrapSteps) * nr, st), "batch phase")) != FSE_OK) return s;
     }
     if ((s = chk(launch_colb<COL_KIN2>(P->ny, ck, mk1, twy, ddesc, nr, 0, st), "batch kinetic")) != FSE_OK)
       return s;
-    if ((s = chk(launch_xb(XP_INV, P->nx, xa, twn, tw2n, ddesc, nr, t0, nsteps, st), "batch x")) != FSE_OK) return s;
+    if ((s = chk(launch_xb(XP_INV, P->nx, xa, twn, tw2n, ddesc, nr, trap, st), "batch x")) != FSE_OK) return s;
     if (multi) {
       cudaError_t e = cudaEventRecord(B->gdone[gi], st);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(st0, B->gdone[gi], 0);
@@ -308,8 +314,9 @@ fse_status fse_batch_step(fse_batch_t B, void* const* psi, double t0, int nsteps
       d.spec = k == 0 ? P->ws_ptr(P->off_spec) : B->ptr(B->off_spec[r]);
       d.kin_half = k == 0 ? P->ws_ptr(P->off_kin_half) : B->ptr(B->off_kh[r]);
       d.kin_full = k == 0 ? P->ws_ptr(P->off_kin_full) : B->ptr(B->off_kf[r]);
-      d.beta = p.beta;
-      d.lam = p.lambda;
+      d.beta_dt = (float)(p.beta * p.dt);
+      d.lam = (float)p.lambda;
+      d.a0 = (float)(p.dt * (1.0 / (4.0 * P->nx * P->ny)));
       d.dt = p.dt;
       d.omega = p.omega;
       d.gx2 = p.gamma[0] * p.gamma[0];
