@@ -12,6 +12,7 @@
 // the kernels through device tables uploaded ahead of each replay.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>

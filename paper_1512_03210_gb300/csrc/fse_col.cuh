@@ -145,7 +145,7 @@ struct ColCfg {
   static constexpr size_t CHAT = S::KHAT ? sizeof(Real) * (size_t)(N + 1) * NC : 0;
   __host__ __device__ static constexpr size_t smem() { return EXCH + CHAT; }
   // registers: 128 per thread for 16 float pairs (64 data registers) and the
-  // float64 passes with eight elements, 96 up to 12 elements, 80 or 64 below
+  // float64 passes with eight elements, 96 up to 12 elements, 80 or 64 below.
   __host__ __device__ static constexpr int minb() {
     const int thr = E > 12 || (sizeof(Real) == 8 && E > 6) ? 512
                                                            : (E > 8 || sizeof(Real) == 8 || VAR == COL_LZ ? 640 : (S::KHAT ? 768 : 1024));
@@ -416,12 +416,12 @@ __device__ __forceinline__ void col_tile(const ColArgs& a, const MulArgs& m, con
       t *= su.inv * sd.inv;
       t = block_sum(t, red);
       if (tid == 0) a.part[bid] = t;
-      return;
-    }
+    } else {
 #pragma unroll
-    for (int q = 0; q < CW; ++q) geo.p[q] = reinterpret_cast<C*>(a.out) + (geo.p[q] - reinterpret_cast<C*>(a.data));
-    geo.vec = geo.vec && (reinterpret_cast<uintptr_t>(geo.p[0]) % 16 == 0);
-    F::template each<RF>(it, [&](int e, int row, int) { col_st(geo, row * ls, v[e]); });
+      for (int q = 0; q < CW; ++q) geo.p[q] = reinterpret_cast<C*>(a.out) + (geo.p[q] - reinterpret_cast<C*>(a.data));
+      geo.vec = geo.vec && (reinterpret_cast<uintptr_t>(geo.p[0]) % 16 == 0);
+      F::template each<RF>(it, [&](int e, int row, int) { col_st(geo, row * ls, v[e]); });
+    }
   } else if constexpr (K::S::KIN) {
     F::template each<RF>(it, [&](int e, int row, int) { v[e] = col_ld(geo, row * ls); });
     F::template run<-1, true, false, false>(v, buf, addr, tw, it);

@@ -54,18 +54,13 @@ struct XArgs {
   } f;
 };
 
-// the step-dependent scalars of an x pass (phase coefficients)
-__host__ __device__ inline void fill_f32_phase(XArgs& a) {
+__host__ __device__ inline void fill_f32(XArgs& a) {
   a.f.beta_dt = (float)a.beta_dt;
   a.f.lam = (float)a.lam;
   a.f.pa = (float)a.pa;
   a.f.pb = (float)a.pb;
   a.f.pc = (float)a.pc;
   a.f.pe = (float)a.pe;
-}
-
-__host__ __device__ inline void fill_f32(XArgs& a) {
-  fill_f32_phase(a);
   a.f.lo0 = (float)a.lo0;
   a.f.lo1 = (float)a.lo1;
   a.f.lo2 = (float)a.lo2;
@@ -410,7 +405,7 @@ template <> __device__ __forceinline__ double sin_sq(double v) {
 // Window integral of the optical lattice at the point (X, Y, Z) of the rotating
 // frame (Gauss-Legendre nodes of the window in a.lat_*).
 template <typename Real>
-__device__ __noinline__ Real lattice_integral(const XArgs& a, Real X, Real Y, Real Z) {
+__device__ __forceinline__ Real lattice_integral(const XArgs& a, Real X, Real Y, Real Z) {
   const Real kx = prm<Real>(a.lat_k[0], a.f.lat_k[0]), ky = prm<Real>(a.lat_k[1], a.f.lat_k[1]);
   const Real kz = prm<Real>(a.lat_k[2], a.f.lat_k[2]);
   const Real zt = kz != Real(0) ? sin_sq(kz * Z) : Real(0);
@@ -421,6 +416,11 @@ __device__ __noinline__ Real lattice_integral(const XArgs& a, Real X, Real Y, Re
     acc += prm<Real>(a.lat_w[q], a.f.lat_w[q]) * (sin_sq(kx * xr) + sin_sq(ky * yr) + zt);
   }
   return prm<Real>(a.lat_amp, a.f.lat_amp) * acc;
+}
+// out of line, for the adjoint's unrolled loop (the arguments go through local memory)
+template <typename Real>
+__device__ __noinline__ Real lattice_call(const XArgs& a, Real X, Real Y, Real Z) {
+  return lattice_integral<Real>(a, X, Y, Z);
 }
 
 
@@ -447,7 +447,7 @@ __device__ __forceinline__ LineTrap<Real, CW> line_trap(const XArgs& a, int l) {
   t.c0 = lane_of(c0);
   return t;
 }
-template <typename Real, int CW, bool LAT>
+template <typename Real, int CW, bool LAT, bool INLINE = false>
 __device__ __forceinline__ typename LaneOf<Real>::T trap_phase(const XArgs& a, const LineTrap<Real, CW>& t, int x, bool lat) {
   typedef typename LaneOf<Real>::T L;
   const Real X = fma_rn(prm<Real>(a.h0, a.f.h0), Real(x), prm<Real>(a.lo0, a.f.lo0));
@@ -456,7 +456,7 @@ __device__ __forceinline__ typename LaneOf<Real>::T trap_phase(const XArgs& a, c
   if (LAT && lat) {
     Real v[CW];
 #pragma unroll
-    for (int q = 0; q < CW; ++q) v[q] = lattice_integral<Real>(a, X, t.Y[q], t.Z[q]);
+    for (int q = 0; q < CW; ++q) v[q] = INLINE ? lattice_integral<Real>(a, X, t.Y[q], t.Z[q]) : lattice_call<Real>(a, X, t.Y[q], t.Z[q]);
     P = ladd(P, lane_of(v));
   }
   return P;
@@ -726,12 +726,32 @@ __device__ __forceinline__ void xpass_body(const XArgs& a, const typename TwOf<R
         const L fsc = lbc<L>(rescale ? Real(*a.scale) : Real(1));
         // u1 lies in psi, or in another field (aux)
         const C* u1 = a.aux ? reinterpret_cast<const C*>(a.aux) + (long long)l0 * NX : (const C*)line0;
+        if constexpr (KIND == XP_AL) {
+          // The lattice's window integral in a rolled loop of its own while
+          // nothing else is live. A call per point among the loaded elements
+          // saved and restored their registers, and took its arguments through
+          // local memory (128 x 192 x 24, 4 steps: 502 us; rolled 489, inlined
+          // 475). A thread's points of the field are its own.
+#pragma unroll 1
+          for (int i = 0; i < (NX / F1::RF + T - 1) / T; ++i) {
+            if (!F1::template ok<F1::RF>(it, i)) continue;
+#pragma unroll 1
+            for (int x = it + i * T; x < NX; x += NX / F1::RF)
+              real_st<RS>(field, g, x, lfma(lam, phi_at(x), trap_phase<Real, CW, true, true>(a, trap, x, true)));
+          }
+        }
         Vec<L> v[F1::E];
         F1::template each<F1::RF>(it, [&](int e, int x, int) { v[e] = line_ld<NX>(u1, g, nl, x); });
         F1::template each<F1::RF>(it, [&](int e, int x, int) {
           const Vec<L> u = v[e];
           const L rho = lfma(u.re, u.re, lmul(u.im, u.im));
-          const L th = lfma(bd, rho, lfma(lam, phi_at(x), trap_phase<Real, CW, KIND == XP_AL>(a, trap, x, true)));
+          L th;
+          if constexpr (KIND == XP_AL) {
+            real_ld<RS>(field, g, x, th);
+            th = lfma(bd, rho, th);
+          } else {
+            th = lfma(bd, rho, lfma(lam, phi_at(x), trap_phase<Real, CW, false>(a, trap, x, true)));
+          }
           v[e] = phase_mul(u, th);
           if (rescale) v[e] = {lmul(fsc, v[e].re), lmul(fsc, v[e].im)};
         });
