@@ -250,7 +250,8 @@ fse_status fse_batch_precompute(fse_batch_t batch);
  * (float2). The first call with a given nsteps captures its launches (every
  * size group on a stream of its own) into a CUDA graph, on a stream the batch
  * owns; later calls with that nsteps only upload the pointers and t0 and
- * replay the graph. The capture uses thread-local mode, so the first call with
+ * replay the graph; the graphs of 16 step counts are kept, and none when
+ * another workspace is attached. The capture uses thread-local mode, so the first call with
  * a new nsteps must not be made while this thread captures another stream.
  * Asynchronous, ordered on the batch's stream. Errors: FSE_ERR_INVALID (null
  * or misaligned pointers, precompute not run), FSE_ERR_CUDA (capture or

@@ -66,11 +66,19 @@ struct fse_batch {
   std::vector<Graph> graphs;
   cudaStream_t cap = nullptr;
   cudaEvent_t cap_in = nullptr, cap_out = nullptr;
+  // a graph that a replay still uses is freed when that replay has ended
+  // (cuGraphExecDestroy does not end it)
+  void drop_graphs(size_t n) {
+    for (size_t i = 0; i < n; ++i) cudaGraphExecDestroy(graphs[i].exec);
+    graphs.erase(graphs.begin(), graphs.begin() + n);
+  }
   size_t off_t0 = 0;  // device scalar: the call's start time
   char* ptr(size_t off) const { return static_cast<char*>(ws) + off; }
 };
 
 namespace {
+// step counts whose graphs are kept; a further one takes the oldest's place
+constexpr size_t kMaxGraphs = 16;
 size_t al(size_t v) { return (v + 255) & ~(size_t)255; }
 fse_status bfail(fse_batch* B, fse_status st, const std::string& m) {
   B->err = m;
@@ -162,6 +170,8 @@ fse_status fse_batch_set_workspace(fse_batch_t B, void* ptr, size_t bytes) {
   if (!B || !ptr) return FSE_ERR_INVALID;
   if (reinterpret_cast<uintptr_t>(ptr) % 256 != 0) return bfail(B, FSE_ERR_INVALID, "workspace not 256-byte aligned");
   if (bytes < B->ws_bytes) return bfail(B, FSE_ERR_NOMEM, "workspace smaller than fse_batch_create reported");
+  // the captured launches hold addresses of the workspace they were captured with
+  if (ptr != B->ws) B->drop_graphs(B->graphs.size());
   B->ws = ptr;
   B->precomputed = false;
   for (auto& G : B->groups) {
@@ -350,6 +360,7 @@ fse_status fse_batch_step(fse_batch_t B, void* const* psi, double t0, int nsteps
     e = cudaGraphInstantiate(&exec, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return bfail(B, FSE_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+    if (B->graphs.size() >= kMaxGraphs) B->drop_graphs(1);
     B->graphs.push_back({nsteps, exec, nl});
     gr = &B->graphs.back();
   }
@@ -365,7 +376,7 @@ fse_status fse_batch_step(fse_batch_t B, void* const* psi, double t0, int nsteps
 
 fse_status fse_batch_destroy(fse_batch_t B) {
   if (!B) return FSE_OK;
-  for (auto& g : B->graphs) cudaGraphExecDestroy(g.exec);
+  B->drop_graphs(B->graphs.size());
   for (auto& G : B->groups) fse_plan_destroy(G.plan);
   for (cudaStream_t s : B->gstream) cudaStreamDestroy(s);
   for (cudaEvent_t e : B->gdone) cudaEventDestroy(e);
