@@ -89,11 +89,13 @@ __global__ void __launch_bounds__(256) k_gs_norm(const typename Cplx<Real>::T* a
   if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
-// x <- x / ||x|| with ||x||^2 = hd * norm[0], and (old non-null) partials of max |x - old|
+// x <- x / ||x|| with ||x||^2 = hd * norm[0], and (old non-null) partials of max |x - old|.
+// A norm that is not positive (the host then returns an error) leaves x as it is.
 template <typename Real>
 __global__ void __launch_bounds__(256) k_gs_normalise(typename Cplx<Real>::T* x, const typename Cplx<Real>::T* old,
                                                       const double* norm, double hd, long long N, double* part) {
   __shared__ double red[256];
+  if (!(norm[0] > 0.0)) return;
   const Real f = Real(1.0 / sqrt(hd * norm[0]));
   double m = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
