@@ -297,6 +297,11 @@ XArgs x_args(fse_plan* P, void* psi, void* spec) {
   return a;
 }
 
+// The index along axis j whose coordinate is next to zero.
+int origin_index(const fse_plan* P, int j) {
+  return (int)std::fmin(std::fmax(std::round(-P->p.lo[j] / P->h[j]), 0.0), P->p.n[j] - 1.0);
+}
+
 // Gauss-Legendre nodes of the window [ta, tb] for the lattice integral (Eq.
 // int_poten by quadrature): weights and (cos, sin)(Omega tau_q). Without
 // rotation the integrand is constant in time and one node is exact.

@@ -73,6 +73,7 @@ fse_status col(fse_plan* P, int kind, int n, int var, const ColArgs& a, const Mu
 fse_status xpass(fse_plan* P, int kind, const XArgs& a);
 int x_tiles(fse_plan* P, int nlines);
 XArgs x_args(fse_plan* P, void* psi, void* spec);
+int origin_index(const fse_plan* P, int j);
 void lattice_nodes(fse_plan* P, double ta, double tb, XArgs& a);
 fse_status kinetic_yz(fse_plan* P, void* psi, double f, double dt);
 fse_status nonlocal_yz(fse_plan* P, void* spec, double ta, double tb, bool integrated, const double* mdir,

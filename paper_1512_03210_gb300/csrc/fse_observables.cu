@@ -33,6 +33,9 @@ struct ObsArgs {
   double lo[3], h[3];
   double c, s;   // cos, sin of Omega t
   double lat_amp, lat_k[3];  // optical lattice lat_amp sum_v sin^2(lat_k[v] x_v)
+  int ic[3];     // the moments' origin: the grid index next to the coordinates' zero
+  bool by_points;  // the x, y part of the harmonic trap energy point by point
+  double g2[3];  // gamma_v^2 / 2
 };
 
 // CW points of a line 32 apart (zero past the end)
@@ -49,29 +52,39 @@ __device__ __forceinline__ Vec<typename LaneOf<Real>::T> pair_at(const typename 
   return {lane_of(re), lane_of(im)};
 }
 
-// lattice energy of a lane's points of a line
-template <typename C> __device__ __forceinline__ double lattice_line(const C* row, const ObsArgs& o, int iy, int iz, int lane) {
+// energies of a lane's points of a line that are formed in float64 point by
+// point: the lattice's and (by_points) the harmonic trap's along x and y
+template <typename C> __device__ __forceinline__ double potential_line(const C* row, const ObsArgs& o, int iy, int iz, int lane) {
   const double y = o.lo[1] + o.h[1] * iy, z = o.lo[2] + o.h[2] * iz;
   double acc = 0.0;
   for (int x = lane; x < o.nx; x += 32) {
     const C u = row[x];
     const double rho = (double)u.x * u.x + (double)u.y * u.y, xx = o.lo[0] + o.h[0] * x;
-    const double sx = sin(o.lat_k[0] * (o.c * xx + o.s * y)), sy = sin(o.lat_k[1] * (-o.s * xx + o.c * y)),
-                 sz = sin(o.lat_k[2] * z);
-    acc += o.lat_amp * (sx * sx + sy * sy + sz * sz) * rho;
+    const double X = o.c * xx + o.s * y, Y = -o.s * xx + o.c * y;
+    double w = 0.0;
+    if (o.by_points) w = o.g2[0] * X * X + o.g2[1] * Y * Y;
+    if (o.lat_amp != 0.0) {
+      const double sx = sin(o.lat_k[0] * X), sy = sin(o.lat_k[1] * Y), sz = sin(o.lat_k[2] * z);
+      w += o.lat_amp * (sx * sx + sy * sy + sz * sz);
+    }
+    acc += w * rho;
   }
   return acc;
 }
 
-// Moments of the density, one warp per line, in index units from the grid's
-// middle (exact): along a line only the sums of rho, rho^2, rho i and rho i^2
-// are formed, and a line's y and z enter once; the coordinates and the harmonic
-// trap energy follow from the sums on the host. In float64 that is about 11
+// Moments of the density, one warp per line, in index units from the index next
+// to the coordinates' zero: along a line only the sums of rho, rho^2, rho i and
+// rho i^2 are formed, and a line's y and z enter once; the coordinates and the
+// harmonic trap energy follow from the sums on the host. From that origin the
+// terms of x = c + h i and x^2 = c^2 + 2 c h i + h^2 i^2 have one sign, or c is
+// within half a spacing of zero (their moduli then add up to nine times x^2 at
+// most). From the grid's middle they cancel in a box to one side of zero: x^2
+// of a cloud at 0.5 in [0, 16] was 5e-14 off, now 1e-16. In float64 that is about 11
 // slots of the FP64 pipe per point in place of 45 (128^3 float32 fields: 172 ->
 // 56 us, the pipe's time); float fields are summed by three floats (ExactSum):
 // 33 us, the chains of two-sums of the 16 warps that 126 registers leave an SM.
-// Slots: rho, rho^2, lattice energy, and rho times i, j, k, i i, j j, k k, i j.
-__global__ void __launch_bounds__(256) k_obs_phys(const float2* __restrict__ psi, ObsArgs o, int nz, double* part) {
+// Slots: rho, rho^2, point energies, and rho times i, j, k, i i, j j, k k, i j.
+__global__ void __launch_bounds__(256) k_obs_phys(const float2* __restrict__ psi, ObsArgs o, double* part) {
   __shared__ double red[10 * 256];
   typedef ExactSum<float2> Sum;
   const int lane = threadIdx.x & 31, nw = gridDim.x * 8;
@@ -97,15 +110,15 @@ __global__ void __launch_bounds__(256) k_obs_phys(const float2* __restrict__ psi
     for (int x = lane; x < o.nx; x += 64) {
       const Vec<float2> u = pair_at<float>(row, x, o.nx);
       const Sum rho = Sum::density(lmul(su.scale, u.re), lmul(su.scale, u.im));
-      const float i = (float)(x - o.nx / 2);
+      const float i = (float)(x - o.ic[0]);
       const float2 i2 = make_float2(i, i + 32.f);
       s0.add(rho);
       s1.prod(i2, rho);
       tii.prod(lmul(i2, i2), rho);
       t1.square(rho);
     }
-    if (o.lat_amp != 0.0) lat += lattice_line(row, o, iy, iz, lane);
-    const float j = (float)(iy - o.ny / 2), k = (float)(iz - nz / 2);
+    if (o.by_points || o.lat_amp != 0.0) lat += potential_line(row, o, iy, iz, lane);
+    const float j = (float)(iy - o.ic[1]), k = (float)(iz - o.ic[2]);
     const float2 j2 = make_float2(j, j), k2 = make_float2(k, k);
     t0.add(s0);
     ti.add(s1);
@@ -121,15 +134,14 @@ __global__ void __launch_bounds__(256) k_obs_phys(const float2* __restrict__ psi
   block_sums(acc, red, [&](int k, double v) { part[k * kPartStride + blockIdx.x] = v; });
 }
 
-__global__ void __launch_bounds__(256) k_obs_phys(const double2* __restrict__ psi, ObsArgs o, int nz,
-                                                  double* part) {
+__global__ void __launch_bounds__(256) k_obs_phys(const double2* __restrict__ psi, ObsArgs o, double* part) {
   __shared__ double red[10 * 256];
   const int lane = threadIdx.x & 31, nw = gridDim.x * 8;
   double acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   for (int l = blockIdx.x * 8 + (threadIdx.x >> 5); l < o.nlines; l += nw) {
     const double2* row = psi + (long long)l * o.nx;
     const int iy = l % o.ny, iz = l / o.ny;
-    double s0 = 0.0, s1 = 0.0, i0 = lane - o.nx / 2;
+    double s0 = 0.0, s1 = 0.0, i0 = lane - o.ic[0];
 #pragma unroll 4
     for (int x = lane; x < o.nx; x += 32, i0 += 32.0) {
       const double2 u = row[x];
@@ -139,8 +151,8 @@ __global__ void __launch_bounds__(256) k_obs_phys(const double2* __restrict__ ps
       s1 += t;
       acc[6] = fma(t, i0, acc[6]);
     }
-    if (o.lat_amp != 0.0) acc[2] += lattice_line(row, o, iy, iz, lane);
-    const double j = iy - o.ny / 2, k = iz - nz / 2, a = j * s0, b = k * s0;
+    if (o.by_points || o.lat_amp != 0.0) acc[2] += potential_line(row, o, iy, iz, lane);
+    const double j = iy - o.ic[1], k = iz - o.ic[2], a = j * s0, b = k * s0;
     acc[0] += s0;
     acc[3] += s1;
     acc[4] += a;
@@ -328,16 +340,21 @@ fse_status observables(fse_plan* P, const void* psi_in, double t, const double* 
   o.nx = P->nx;
   o.ny = P->ny;
   o.nlines = P->ny * P->nz;
-  double g2[3];  // gamma_v^2 / 2
   for (int j = 0; j < 3; ++j) {
     o.lo[j] = j < P->dim ? P->p.lo[j] : 0.0;
     o.h[j] = P->h[j];
     const double g = j < P->dim ? (gam ? gam[j] : P->p.gamma[j]) : 0.0;
-    g2[j] = 0.5 * g * g;
+    o.g2[j] = 0.5 * g * g;
+    o.ic[j] = j < P->dim ? origin_index(P, j) : 0;
     o.lat_k[j] = j < P->dim ? P->p.lat_k[j] : 0.0;
   }
   o.c = std::cos(P->p.omega * t);
   o.s = std::sin(P->p.omega * t);
+  // In a turned frame the moments give a trap's energy up to rounding of that of
+  // its stiff axis in all directions: for a cloud along the soft axis of frequencies
+  // 100 : 1 it was 6e-14 off, summed point by point 1e-16, as it is beyond 2 : 1.
+  const double stiff = std::fmax(o.g2[0], o.g2[1]), soft = std::fmin(o.g2[0], o.g2[1]);
+  o.by_points = o.s != 0.0 && !(stiff <= 4.0 * soft);
   o.lat_amp = P->p.lat_amp;
   const long long N = (long long)P->nx * P->ny * P->nz;
   const int blocks = std::min(2 * kSMs, (o.nlines + 7) / 8);
@@ -362,7 +379,7 @@ fse_status observables(fse_plan* P, const void* psi_in, double t, const double* 
   }
 
   cudaEvent_t ev = prof_begin(P);
-  k_obs_phys<<<blocks, 256, 0, P->stream>>>(psi, o, P->nz, part);
+  k_obs_phys<<<blocks, 256, 0, P->stream>>>(psi, o, part);
   prof_end(P, FSE_PASS_OTHER, ev);
   if ((st = launched(P, cudaGetLastError(), "observables")) != FSE_OK) return st;
   for (int k = SL_MASS; k <= SL_XY; ++k) cnt.n[k] = blocks;
@@ -416,11 +433,10 @@ fse_status observables(fse_plan* P, const void* psi_in, double t, const double* 
 
   double hd = 1.0;
   for (int j = 0; j < P->dim; ++j) hd *= P->h[j];
-  // sums in index units from the middle -> coordinates x = c + h i
+  // sums in index units -> coordinates x = c + h i
   {
-    const int n3[3] = {P->nx, P->ny, P->nz};
     double c[3];
-    for (int j = 0; j < 3; ++j) c[j] = j < P->dim ? o.lo[j] + o.h[j] * (n3[j] / 2) : 0.0;
+    for (int j = 0; j < 3; ++j) c[j] = j < P->dim ? o.lo[j] + o.h[j] * o.ic[j] : 0.0;
     const double s0 = h[SL_MASS], i1[3] = {h[SL_X], h[SL_Y], h[SL_Z]};
     h[SL_XY] = c[0] * c[1] * s0 + c[0] * o.h[1] * i1[1] + c[1] * o.h[0] * i1[0] + o.h[0] * o.h[1] * h[SL_XY];
     for (int j = 0; j < 3; ++j) {
@@ -432,8 +448,11 @@ fse_status observables(fse_plan* P, const void* psi_in, double t, const double* 
   out->mass = hd * h[SL_MASS];
   out->e_kin = 0.5 * hd / (double)N * h[SL_KIN];
   // W = g2_x X^2 + g2_y Y^2 + g2_z z^2 (+ lattice), X = c x + s y, Y = -s x + c y
-  out->e_pot = hd * (h[SL_WRHO] + g2[0] * (o.c * o.c * h[SL_XX] + 2 * o.c * o.s * h[SL_XY] + o.s * o.s * h[SL_YY]) +
-                     g2[1] * (o.s * o.s * h[SL_XX] - 2 * o.c * o.s * h[SL_XY] + o.c * o.c * h[SL_YY]) + g2[2] * h[SL_ZZ]);
+  double trap = o.g2[2] * h[SL_ZZ];
+  if (!o.by_points)
+    trap += o.g2[0] * (o.c * o.c * h[SL_XX] + 2 * o.c * o.s * h[SL_XY] + o.s * o.s * h[SL_YY]) +
+            o.g2[1] * (o.s * o.s * h[SL_XX] - 2 * o.c * o.s * h[SL_XY] + o.c * o.c * h[SL_YY]);
+  out->e_pot = hd * (h[SL_WRHO] + trap);
   out->e_int = 0.5 * P->p.beta * hd * h[SL_RHO2];
   out->e_non = has_nonlocal(P) ? 0.5 * P->p.lambda * hd * h[SL_NON] : 0.0;
   out->lz = hd * (h[SL_LZY] + h[SL_LZX]);
