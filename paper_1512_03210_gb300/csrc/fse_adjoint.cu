@@ -43,6 +43,7 @@ XArgs adjoint_args(fse_plan* P, void* g, void* spec, const void* u1, double ta, 
   trap_coefficients(P, ta, tb, gamma, pc);
   XArgs x = x_args(P, g, spec);
   x.aux = u1;
+  x.ix0 = origin_index(P, 0);
   x.beta_dt = P->p.beta * P->p.dt;
   x.lam = P->p.lambda;
   x.pa = pc[0];

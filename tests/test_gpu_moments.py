@@ -78,3 +78,24 @@ def test_trap_energy_in_a_turned_frame(lib, gamma, prec):
     # points: X is off by 2 (|c x| + |s y|) / |X| = 36 units, its square by twice that, and 64 for the
     # sum; moments (up to 2 : 1): 36 units for terms that add up to four times the energy
     assert abs(plan.observables(psi, t)["e_pot"] - ref) <= 144 * 2.0**-53 * ref
+
+
+@pytest.mark.parametrize("sweep", [False, True])
+@pytest.mark.parametrize("name", sorted(BOXES))
+def test_trap_gradient_off_the_origin(lib, name, sweep):
+    """With a step of 1e-18 the kinetic factors are 1 to 1e-15 and the phase vanishes:
+    dJ/dgamma_v = gamma_v dt sum_x x_v^2 Im(conj(g) psi), one-signed for g = -i psi."""
+    n, lo, hi, centre, width = BOXES[name]
+    d = dict(_params(n, "f64", lo, hi, (1.0, 1.2, 2.0)[:len(n)]), beta=0.0, dt=1e-18)
+    plan = lib.Plan(d)
+    psi = plan.to_device(_cloud(d, centre, width))
+    g = psi * -1j
+    if sweep:
+        dg = plan.adjoint_sweep(psi, g, 0.0, np.array([d["gamma"]]))[0]
+    else:
+        dg = plan.adjoint(psi, g, 0.0, None, want_dgamma=True)
+    u = psi.cpu().numpy()
+    rho = u.real.astype(LD) ** 2 + u.imag.astype(LD) ** 2
+    for v, x in enumerate(_axes(d)):
+        ref = float(LD(d["gamma"][v]) * LD(1e-18) * np.sum(x * x * rho))
+        assert abs(dg[v] - ref) <= EPS * ref, (v, dg[v], ref, dg[v] / ref - 1)
