@@ -422,6 +422,12 @@ fse_status nonlocal_yz(fse_plan* P, void* spec, double ta, double tb, bool integ
     m.q[3] = 2 * c * M[3] * dk[0] * dk[1];
     m.q[4] = 2 * c * M[4] * dk[0] * dk[2];
     m.q[5] = 2 * c * M[5] * dk[1] * dk[2];
+    // The two terms nearly cancel over the modes, so a float plan rounds them
+    // alike: the factors q keep their tails and follow a0's rounding (1/3 of a
+    // grid with a factor of three is 3e-8 off; alone in a0 that was 2e-7 of the
+    // field energy of a 64 x 32 x 48 cloud).
+    if (P->prec == FSE_F32 && m.a0 != 0.0)
+      for (double& q : m.q) q *= (double)(float)m.a0 / m.a0;
   }
   ColArgs ag{spec, P->sx, (long long)2 * P->ny * P->sx, 2 * P->ny, P->nx + 1};
   if ((st = col(P, FSE_PASS_KHAT, P->nz, COL_KHAT, ag, m)) != FSE_OK) return st;

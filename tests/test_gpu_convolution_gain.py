@@ -28,3 +28,19 @@ def test_round_trip_of_a_white_density(lib, n):
     gain = o["e_non"] / (-0.1 * o["e_int"]) - 1
     print(f"{n}: {gain:.2e}")
     assert abs(gain) <= 8e-9
+
+
+@pytest.mark.parametrize("n", [(64, 32, 48), (96, 64, 64), (32, 48, 128)])
+def test_dipolar_terms_are_rounded_alike(lib, n):
+    """N has one factor of three, so that -1 / (8 N) is 2.98e-8 off as a float. Over a
+    white spectrum the dipolar kernel's two terms nearly cancel, and with them every
+    gain that they share; an error of the first term alone stays whole. A quarter of it
+    is the bound."""
+    axis = dict(dip_n=(0.6, 0.0, 0.8))
+    rng = np.random.default_rng(2)
+    psi = (rng.standard_normal(n[::-1]) + 1j * rng.standard_normal(n[::-1])).astype(np.complex64)
+    a, b = _plan(lib, n, **axis), _plan(lib, n, "f64", **axis)
+    oa, ob = a.observables(a.to_device(psi), 0.0), b.observables(b.to_device(psi), 0.0)
+    err = (oa["e_non"] - ob["e_non"]) / (0.1 * ob["e_int"])
+    print(f"{n}: {err:.2e}, kernel mean {ob['e_non'] / (0.1 * ob['e_int']):.2f}")
+    assert abs(err) <= 2.98e-8 / 4
