@@ -248,6 +248,8 @@ def fse_step_adjoint(plan, psi_n, g, t_n: float, gamma_n=None, want_dgamma: bool
 def fse_adjoint_sweep(plan, psi_0, states, g, t0: float, gammas, dim: int) -> np.ndarray:
     """Pulls g back (in place) through len(gammas) steps from psi_0; returns dJ/dgamma [nsteps][dim]."""
     keep, gp = _gammas(gammas)
+    if keep is None or keep.ndim != 2 or keep.shape[1] != dim:
+        raise ValueError(f"fse_adjoint_sweep: gammas must be [nsteps][{dim}]")
     dg = np.zeros((len(keep), dim), dtype=np.float64)
     _check(load().fse_adjoint_sweep(plan, _ptr(psi_0), _ptr(states), _ptr(g), float(t0), len(keep), gp,
                                     dg.ctypes.data_as(ct.c_void_p)), "fse_adjoint_sweep", plan)
