@@ -41,24 +41,30 @@ __device__ __forceinline__ void round_pair(double c, double s, double2* out) { *
 // value are exact to rounding.
 __device__ __forceinline__ double2 tan_pair(double c, double s) {
   if (fabs(c) < 1e-30) return make_double2(1e-40, s * 1e40);
-  const double t0 = s / c, rest = fma(-t0, c, s) / c;  // tangent and the remainder of its rounding
+  if (s == 0.0) return make_double2(c, s * c);
+  const double ic = 1.0 / c, t1 = s * ic, t0 = fma(fma(-t1, c, s), ic, t1);
+  const double rest = fma(-t0, c, s) * ic;  // the remainder of the tangent's rounding
+  // (c^2 (1 + t0^2) - 1) / 2 with the rounding errors of its products and sum; a
+  // neighbour changes it by dc / c and t0 dt / (1 + t0^2), with 1 + t0^2 = 1 / c^2
+  const double p = t0 * t0, pe = fma(t0, t0, -p);
+  const double q = 1.0 + p, z = q - p, qe = (1.0 - z) + (p - (q - z)) + pe;
+  const double a = c * c, ae = fma(c, c, -a);
+  const double m = a * q, me = fma(a, q, -m) + a * qe + ae * q;
+  const double e0 = ((m - 1.0) + me) * 0.5;
   double best = 1e300;
   double2 r = make_double2(c, t0);
-  for (int i = -1; i <= 1; ++i)
-    for (int j = -1; j <= 1; ++j) {
-      const double cc = i == 0 ? c : nextafter(c, i < 0 ? -2.0 : 2.0);
-      const double tt = j == 0 ? t0 : nextafter(t0, j < 0 ? -1e300 : 1e300);
-      // cc^2 (1 + tt^2) - 1 with the rounding errors of its products and sum
-      const double p = tt * tt, pe = fma(tt, tt, -p);
-      const double q = 1.0 + p, z = q - p, qe = (1.0 - z) + (p - (q - z)) + pe;
-      const double a = cc * cc, ae = fma(cc, cc, -a);
-      const double m = a * q, me = fma(a, q, -m) + a * qe + ae * q;
-      const double cost = fabs(((m - 1.0) + me) * 0.5) + fabs((tt - t0) - rest) / q;
+  for (int j = -1; j <= 1; ++j) {
+    const double tt = __longlong_as_double(__double_as_longlong(t0) + j), dt = tt - t0;
+    const double e = fma(t0 * a, dt, e0), turn = fabs(dt - rest) * a;
+    for (int i = -1; i <= 1; ++i) {
+      const double cc = __longlong_as_double(__double_as_longlong(c) + i);
+      const double cost = fabs(fma(cc - c, ic, e)) + turn;
       if (cost < best) {
         best = cost;
         r = make_double2(cc, tt);
       }
     }
+  }
   return r;
 }
 
