@@ -229,9 +229,8 @@ static cudaError_t gs_fwd_launch(const GsFwd& a, const void* twn, cudaStream_t s
                        : allow_smem(k_gs_fwd<Real, NX, LN, false>, K::smem(), done0);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (a.nlines + LN - 1) / LN;
-  const bool pdl = launch_early<Real>(blocks, NX <= 64);
-  return a.dy ? launch_pass_if(pdl, k_gs_fwd<Real, NX, LN, true>, blocks, K::NT, K::smem(), st, a, reinterpret_cast<W>(twn))
-              : launch_pass_if(pdl, k_gs_fwd<Real, NX, LN, false>, blocks, K::NT, K::smem(), st, a, reinterpret_cast<W>(twn));
+  return a.dy ? launch_pass(k_gs_fwd<Real, NX, LN, true>, blocks, K::NT, K::smem(), st, a, reinterpret_cast<W>(twn))
+              : launch_pass(k_gs_fwd<Real, NX, LN, false>, blocks, K::NT, K::smem(), st, a, reinterpret_cast<W>(twn));
 }
 template <typename Real, int NX, int LN>
 static cudaError_t gs_inv_launch(const GsInv& a, const void* twn, cudaStream_t st) {
@@ -241,7 +240,7 @@ static cudaError_t gs_inv_launch(const GsInv& a, const void* twn, cudaStream_t s
   cudaError_t e = allow_smem(k_gs_inv<Real, NX, LN>, smem, done);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (a.nlines + LN - 1) / LN;
-  return launch_pass_if(launch_early<Real>(blocks, NX <= 64), k_gs_inv<Real, NX, LN>, blocks, K::NT, smem, st, a,
+  return launch_pass(k_gs_inv<Real, NX, LN>, blocks, K::NT, smem, st, a,
                      reinterpret_cast<const typename TwOf<Real>::T*>(twn));
 }
 template <typename Real> cudaError_t launch_gs_fwd(int nx, const GsFwd& a, const void* twn, cudaStream_t st) {

@@ -14,7 +14,7 @@ namespace fse {
 // Launch of a step pass with programmatic dependent launch on the previous
 // kernel in the stream (see pass_prologue).
 template <typename... Params, typename... Args>
-static cudaError_t launch_pass_if(bool pdl, void (*kernel)(Params...), unsigned blocks, unsigned threads, size_t smem,
+static cudaError_t launch_pass(void (*kernel)(Params...), unsigned blocks, unsigned threads, size_t smem,
                                cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks);
@@ -23,29 +23,10 @@ static cudaError_t launch_pass_if(bool pdl, void (*kernel)(Params...), unsigned 
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = pdl;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-template <typename... Params, typename... Args>
-static cudaError_t launch_pass(void (*kernel)(Params...), unsigned blocks, unsigned threads, size_t smem,
-                               cudaStream_t st, Args... args) {
-  return launch_pass_if(true, kernel, blocks, threads, smem, st, args...);
-}
-
-// A float64 pass of one to four tiles per SM is not launched early: its blocks
-// would be dealt to the SMs while the previous pass's still sit there unevenly,
-// and the SM that gets one too many sets the time of a pass bound by the FP64
-// pipe (ground state on 512^2: inverse x pass 47 us early, 25 us after). Light
-// passes, those of the wave function alone along short axes, are over before that
-// counts, and the launch gaps are what they save (shift of 32^3: 55 us after, 49
-// early; ground state of 64^3 8.90 ms and 8.30). Their limits: 64 points; 48 for
-// the forward . factors . inverse of the ground state (rotating, 64^3: 13.7 ms
-// after, 14.1 early). At 48 points and more the density's passes lose with an
-// early launch (a step of 48^3 316 us after, 440 early).
-template <typename Real> static bool launch_early(long long blocks, bool light) {
-  return sizeof(Real) == 4 || light || blocks < kSMs || blocks >= 4 * kSMs;
 }
 
 // cudaFuncSetAttribute once per kernel and device when the dynamic tile comes
@@ -76,8 +57,7 @@ static cudaError_t col_launch(const ColArgs& a, const MulArgs& m, long long bloc
   if (a.blocks_out) *a.blocks_out = (int)blocks;
   MulArgs mf = m;
   fill_f32(mf);
-  constexpr bool light = VAR == COL_RMUL ? N <= 48 : N <= 64 && !K::S::TWO && !K::S::KIN;
-  return launch_pass_if(launch_early<Real>(blocks, light), k_col<Real, N, VAR, NP>, (unsigned)blocks, K::NT, K::smem(), st, a, mf,
+  return launch_pass(k_col<Real, N, VAR, NP>, (unsigned)blocks, K::NT, K::smem(), st, a, mf,
                      reinterpret_cast<const C*>(tw));
 }
 
@@ -130,8 +110,7 @@ static cudaError_t x_launch(const XArgs& a, const void* twn, const void* tw2n, c
   if (blocks <= 0) return cudaSuccess;
   XArgs af = a;
   fill_f32(af);
-  constexpr bool light = NX <= 64 && (KIND == XP_FWD || KIND == XP_INV);
-  return launch_pass_if(launch_early<Real>(blocks, light), k_xpass<Real, NX, LN, KIND>, (unsigned)blocks, K::NT, K::smem(), st, af,
+  return launch_pass(k_xpass<Real, NX, LN, KIND>, (unsigned)blocks, K::NT, K::smem(), st, af,
                      reinterpret_cast<const C*>(twn), reinterpret_cast<const C*>(tw2n));
 }
 
