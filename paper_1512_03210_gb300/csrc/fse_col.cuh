@@ -228,6 +228,21 @@ __device__ __forceinline__ double lane_of(const double (&v)[1]) { return v[0]; }
 __device__ __forceinline__ float2 lane_ld(const float* p) { return *reinterpret_cast<const float2*>(p); }
 __device__ __forceinline__ double lane_ld(const double* p) { return *p; }
 
+// Head and tail: the exact product of two lanes, and sums good to the square of
+// the rounding unit.
+template <typename L> struct Two {
+  L h, l;
+};
+template <typename L> __device__ __forceinline__ Two<L> two_prod(L a, L b) {
+  const L p = lmul(a, b);
+  return {p, lfma(a, b, lneg(p))};
+}
+template <typename L> __device__ __forceinline__ Two<L> two_sum(const Two<L>& a, const Two<L>& b) {
+  const L s = ladd(a.h, b.h), v = lsub(s, a.h);
+  const L e = ladd(lsub(a.h, lsub(s, v)), lsub(b.h, v));
+  return {s, ladd(e, ladd(a.l, b.l))};
+}
+
 // s += Im(conj(u) d), u scaled by su and d by sd
 template <typename L>
 __device__ __forceinline__ void lz_add(const Vec<L>& u, const Vec<L>& d, const L& su, const L& sd, ExactSum<L>& s) {
@@ -462,25 +477,39 @@ __device__ __forceinline__ void col_tile(const ColArgs& a, const MulArgs& m, con
     addr.sync();
     fresh();
     const bool ddi = m.mode == MUL_DDI;
-    // integer frequencies: the spacings are in the factors q, and a float plan
-    // adds what rounding them left (a factor 6e-8 off would act on every mode
-    // alike, and the dipolar energy is a small difference of the modes' sums)
-    Real Aq[CW], Bq[CW];
+    // integer frequencies: the spacings are in the factors q. A and B are one
+    // value for a column, and the dipolar energy is a small difference of sums over
+    // all modes: float plans form both as sums of two floats, with what rounding the
+    // factors left, and A's tail goes on to the elements (rounded in every product
+    // the columns alone left 1e-8 to 2e-8 of the two sums in the energy; now 4e-9.
+    // 256^3 3299 us for four steps without the tails of A, 3310 with them)
+    L A = lbc<L>(0.0), B = A, Al = A;
+    if (ddi) {
+      Real kp_[CW], kx_[CW], kpo_[CW], kxo_[CW];
 #pragma unroll
-    for (int q = 0; q < CW; ++q) {
-      const Real kp = m.lp ? Real(wrap_index(geo.plane[q], m.lp)) : Real(0);
-      const Real kpo = (m.lp && 2 * geo.plane[q] == m.lp) ? Real(0) : kp;
-      const Real kx = Real(geo.px[q]);
-      const Real kxo = (2 * geo.px[q] == m.lx) ? Real(0) : kx;
-      Aq[q] = prm<Real>(m.q[0], m.f.q[0]) * kx * kx + prm<Real>(m.q[1], m.f.q[1]) * kp * kp +
-              prm<Real>(m.q[3], m.f.q[3]) * kxo * kpo;
-      Bq[q] = prm<Real>(m.q[4], m.f.q[4]) * kxo + prm<Real>(m.q[5], m.f.q[5]) * kpo;
+      for (int q = 0; q < CW; ++q) {
+        kp_[q] = m.lp ? Real(wrap_index(geo.plane[q], m.lp)) : Real(0);
+        kpo_[q] = (m.lp && 2 * geo.plane[q] == m.lp) ? Real(0) : kp_[q];
+        kx_[q] = Real(geo.px[q]);
+        kxo_[q] = (2 * geo.px[q] == m.lx) ? Real(0) : kx_[q];
+      }
+      const L kp = lane_of(kp_), kx = lane_of(kx_), kpo = lane_of(kpo_), kxo = lane_of(kxo_);
+      const L xx = lmul(kx, kx), pp = lmul(kp, kp), xp = lmul(kxo, kpo);  // (exact)
+      auto q = [&](int i) { return lbc<L>(prm<Real>(m.q[i], m.f.q[i])); };
       if constexpr (sizeof(Real) == 4) {
-        Aq[q] += m.f.qt[0] * kx * kx + m.f.qt[1] * kp * kp + m.f.qt[3] * kxo * kpo;
-        Bq[q] += m.f.qt[4] * kxo + m.f.qt[5] * kpo;
+        auto t = [&](int i) { return lbc<L>(m.f.qt[i]); };
+        const Two<L> a = two_sum(two_sum(two_prod(q(0), xx), two_prod(q(1), pp)), two_prod(q(3), xp));
+        const L al = lfma(t(0), xx, lfma(t(1), pp, lfma(t(3), xp, a.l)));
+        A = ladd(a.h, al);
+        Al = lsub(al, lsub(A, a.h));
+        const Two<L> b = two_sum(two_prod(q(4), kxo), two_prod(q(5), kpo));
+        B = ladd(b.h, lfma(t(4), kxo, lfma(t(5), kpo, b.l)));
+      } else {
+        A = lfma(q(0), xx, lfma(q(1), pp, lmul(q(3), xp)));
+        B = lfma(q(4), kxo, lmul(q(5), kpo));
       }
     }
-    const L A = lane_of(Aq), B = lane_of(Bq), a0 = lbc<L>(prm<Real>(m.a0, m.f.a0));
+    const L a0 = lbc<L>(prm<Real>(m.a0, m.f.a0));
     const L q2 = lbc<L>(prm<Real>(m.q[2], m.f.q[2]));
     F::template each<RL>(it, [&](int e, int row, int r) {
       // signed frequency of the row: row - M from M/2 on
@@ -491,7 +520,9 @@ __device__ __forceinline__ void col_tile(const ColArgs& a, const MulArgs& m, con
         const L kr = lbc<L>(Real(row - r * (M / RL)) + Real(r * (M / RL) - (up ? M : 0)));
         L b = 2 * row == M ? lbc<L>(0.0) : B;
         if constexpr (sizeof(Real) == 4) b = lfma(lbc<L>(m.f.qt[2]), kr, b);
-        const L f = lfma(lfma(kr, lfma(q2, kr, b), A), cv, a0);
+        L f0 = a0;
+        if constexpr (sizeof(Real) == 4) f0 = lfma(Al, cv, a0);
+        const L f = lfma(lfma(kr, lfma(q2, kr, b), A), cv, f0);
         v[e] = {lmul(f, v[e].re), lmul(f, v[e].im)};
       } else {
         const L f = lmul(a0, cv);
