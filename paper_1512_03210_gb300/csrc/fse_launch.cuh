@@ -101,7 +101,7 @@ cudaError_t launch_col_var(int n, const ColArgs& a, const MulArgs& m, const void
 
 template <typename Real, int NX, int LN, int KIND>
 static cudaError_t x_launch(const XArgs& a, const void* twn, const void* tw2n, cudaStream_t st) {
-  typedef XCfg<Real, NX, LN> K;
+  typedef XLaunch<Real, NX, LN, KIND> K;
   typedef typename TwOf<Real>::T C;
   static std::atomic<unsigned long long> done{0};
   cudaError_t e = allow_smem(k_xpass<Real, NX, LN, KIND>, K::smem(), done);
@@ -110,7 +110,7 @@ static cudaError_t x_launch(const XArgs& a, const void* twn, const void* tw2n, c
   if (blocks <= 0) return cudaSuccess;
   XArgs af = a;
   fill_f32(af);
-  return launch_pass(k_xpass<Real, NX, LN, KIND>, (unsigned)blocks, K::NT, K::smem(), st, af,
+  return launch_pass(k_xpass<Real, NX, LN, KIND>, (unsigned)blocks, K::threads, K::smem(), st, af,
                      reinterpret_cast<const C*>(twn), reinterpret_cast<const C*>(tw2n));
 }
 

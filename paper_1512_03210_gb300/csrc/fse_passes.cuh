@@ -418,6 +418,31 @@ __device__ __forceinline__ Real lattice_integral(const XArgs& a, Real X, Real Y,
   }
   return prm<Real>(a.lat_amp, a.f.lat_amp) * acc;
 }
+// The same for the lanes' points of one x, the nodes' sines of all lanes in one
+// loop.
+template <typename Real, int CW>
+__device__ __forceinline__ void lattice_lanes(const XArgs& a, Real X, const Real (&Y)[CW], const Real (&Z)[CW], Real (&out)[CW]) {
+  const Real kx = prm<Real>(a.lat_k[0], a.f.lat_k[0]), ky = prm<Real>(a.lat_k[1], a.f.lat_k[1]);
+  const Real kz = prm<Real>(a.lat_k[2], a.f.lat_k[2]);
+  Real zt[CW], acc[CW];
+#pragma unroll
+  for (int l = 0; l < CW; ++l) {
+    zt[l] = kz != Real(0) ? sin_sq(kz * Z[l]) : Real(0);
+    acc[l] = Real(0);
+  }
+#pragma unroll 1
+  for (int q = 0; q < a.lat_nq; ++q) {
+    const Real c = prm<Real>(a.lat_c[q], a.f.lat_c[q]), s = prm<Real>(a.lat_s[q], a.f.lat_s[q]);
+    const Real w = prm<Real>(a.lat_w[q], a.f.lat_w[q]);
+#pragma unroll
+    for (int l = 0; l < CW; ++l) {
+      const Real xr = c * X + s * Y[l], yr = -s * X + c * Y[l];
+      acc[l] += w * (sin_sq(kx * xr) + sin_sq(ky * yr) + zt[l]);
+    }
+  }
+#pragma unroll
+  for (int l = 0; l < CW; ++l) out[l] = prm<Real>(a.lat_amp, a.f.lat_amp) * acc[l];
+}
 // out of line, for the adjoint's unrolled loop (the arguments go through local memory)
 template <typename Real>
 __device__ __noinline__ Real lattice_call(const XArgs& a, Real X, Real Y, Real Z) {
@@ -448,7 +473,7 @@ __device__ __forceinline__ LineTrap<Real, CW> line_trap(const XArgs& a, int l) {
   t.c0 = lane_of(c0);
   return t;
 }
-template <typename Real, int CW, bool LAT, bool INLINE = false>
+template <typename Real, int CW, bool LAT>
 __device__ __forceinline__ typename LaneOf<Real>::T trap_phase(const XArgs& a, const LineTrap<Real, CW>& t, int x, bool lat) {
   typedef typename LaneOf<Real>::T L;
   const Real X = fma_rn(prm<Real>(a.h0, a.f.h0), Real(x), prm<Real>(a.lo0, a.f.lo0));
@@ -457,13 +482,28 @@ __device__ __forceinline__ typename LaneOf<Real>::T trap_phase(const XArgs& a, c
   if (LAT && lat) {
     Real v[CW];
 #pragma unroll
-    for (int q = 0; q < CW; ++q) v[q] = INLINE ? lattice_integral<Real>(a, X, t.Y[q], t.Z[q]) : lattice_call<Real>(a, X, t.Y[q], t.Z[q]);
+    for (int q = 0; q < CW; ++q) v[q] = lattice_call<Real>(a, X, t.Y[q], t.Z[q]);
     P = ladd(P, lane_of(v));
   }
   return P;
 }
 __device__ __forceinline__ float lane_get(float2 v, int q) { return q ? v.y : v.x; }
 __device__ __forceinline__ double lane_get(double v, int) { return v; }
+
+// Pass A with a lattice (XP_AL) keeps the lattice's window integrals of a tile's
+// points in shared memory, line by line behind the tile. They depend on nothing
+// that an earlier pass writes and are formed first, while nothing else is live,
+// in narrow tiles by warps that only come for this and leave: the 32 threads of
+// an 8 x 8 or 12 x 8 grid's tile took 13 and 61 us over them. Calls of two steps:
+// 8 x 8 43 -> 28 us, 12 x 8 float64 143 -> 62, 96 x 128 88 -> 56, 512^2 109 -> 86,
+// 128 x 192 x 24 247 -> 154, 512^2 float64 (its sines) 935 -> 913.
+template <typename Real, int NX, int LN, int KIND> struct XLaunch {
+  typedef XCfg<Real, NX, LN> K;
+  static constexpr bool LAT = KIND == XP_AL, HELP = LAT && LN == XWidths<Real, NX>::narrow();
+  static constexpr int threads = HELP && K::NT < 256 ? 256 : K::NT;
+  __host__ __device__ static constexpr size_t smem() { return K::smem() + (LAT ? sizeof(Real) * (size_t)LN * K::RS : 0); }
+  __host__ __device__ static constexpr int minb() { return HELP ? 2 : K::minb(); }
+};
 
 // PDL: the launch is a dependent one (the prologue's wait is here).
 template <typename Real, int NX, int LN, int KIND, bool PDL>
@@ -487,6 +527,25 @@ __device__ __forceinline__ void xpass_body(const XArgs& a, const typename TwOf<R
   const XAddr ad1{g * K::LS1}, ad2{q2 * K::LS2};
   const int l0 = bid * LN, nl = a.nlines - l0;
   C* line0 = reinterpret_cast<C*>(a.psi) + (long long)l0 * NX;
+  Real* lat = reinterpret_cast<Real*>(smem_raw + K::smem());
+  if constexpr (KIND == XP_AL) {
+    typedef XLaunch<Real, NX, LN, KIND> X;
+#pragma unroll 1
+    for (int i = tid; i < K::LP * NX; i += X::threads) {
+      const int h = i / NX, x = i - h * NX;
+      Real Y[CW], Z[CW], v[CW];
+#pragma unroll
+      for (int q = 0; q < CW; ++q) {
+        const int l = l0 + CW * h + q;
+        Y[q] = fma_rn(prm<Real>(a.h1, a.f.h1), Real(l % a.ny), prm<Real>(a.lo1, a.f.lo1));
+        Z[q] = fma_rn(prm<Real>(a.h2, a.f.h2), Real(l / a.ny), prm<Real>(a.lo2, a.f.lo2));
+      }
+      lattice_lanes<Real, CW>(a, fma_rn(prm<Real>(a.h0, a.f.h0), Real(x), prm<Real>(a.lo0, a.f.lo0)), Y, Z, v);
+      real_st<RS>(lat, h, x, lane_of(v));
+    }
+    __syncthreads();
+    if (X::threads > K::NT && tid >= K::NT) return;
+  }
   if constexpr (PDL && LN == XWidths<Real, NX>::narrow() && LN < XWidths<Real, NX>::wide()) {
     // a narrow tile is alone on its SM: its twiddle tables come into L1 before
     // the wait for the previous pass (see col_tile)
@@ -729,32 +788,18 @@ __device__ __forceinline__ void xpass_body(const XArgs& a, const typename TwOf<R
         const L fsc = lbc<L>(rescale ? Real(*a.scale) : Real(1));
         // u1 lies in psi, or in another field (aux)
         const C* u1 = a.aux ? reinterpret_cast<const C*>(a.aux) + (long long)l0 * NX : (const C*)line0;
-        if constexpr (KIND == XP_AL) {
-          // The lattice's window integral in a rolled loop of its own while
-          // nothing else is live. A call per point among the loaded elements
-          // saved and restored their registers, and took its arguments through
-          // local memory (128 x 192 x 24, 4 steps: 502 us; rolled 489, inlined
-          // 475). A thread's points of the field are its own.
-#pragma unroll 1
-          for (int i = 0; i < (NX / F1::RF + T - 1) / T; ++i) {
-            if (!F1::template ok<F1::RF>(it, i)) continue;
-#pragma unroll 1
-            for (int x = it + i * T; x < NX; x += NX / F1::RF)
-              real_st<RS>(field, g, x, lfma(lam, phi_at(x), trap_phase<Real, CW, true, true>(a, trap, x, true)));
-          }
-        }
         Vec<L> v[F1::E];
         F1::template each<F1::RF>(it, [&](int e, int x, int) { v[e] = line_ld<NX>(u1, g, nl, x); });
         F1::template each<F1::RF>(it, [&](int e, int x, int) {
           const Vec<L> u = v[e];
           const L rho = lfma(u.re, u.re, lmul(u.im, u.im));
-          L th;
+          L P = trap_phase<Real, CW, false>(a, trap, x, true);
           if constexpr (KIND == XP_AL) {
-            real_ld<RS>(field, g, x, th);
-            th = lfma(bd, rho, th);
-          } else {
-            th = lfma(bd, rho, lfma(lam, phi_at(x), trap_phase<Real, CW, false>(a, trap, x, true)));
+            L w;
+            real_ld<RS>(lat, g, x, w);
+            P = ladd(P, w);
           }
+          const L th = lfma(bd, rho, lfma(lam, phi_at(x), P));
           v[e] = phase_mul(u, th);
           if (rescale) v[e] = {lmul(fsc, v[e].re), lmul(fsc, v[e].im)};
         });
@@ -768,7 +813,7 @@ __device__ __forceinline__ void xpass_body(const XArgs& a, const typename TwOf<R
 }
 
 template <typename Real, int NX, int LN, int KIND>
-__global__ void __launch_bounds__(XCfg<Real, NX, LN>::NT, XCfg<Real, NX, LN>::minb())
+__global__ void __launch_bounds__(XLaunch<Real, NX, LN, KIND>::threads, XLaunch<Real, NX, LN, KIND>::minb())
 k_xpass(XArgs a, const typename TwOf<Real>::T* __restrict__ twn, const typename TwOf<Real>::T* __restrict__ tw2n) {
   xpass_body<Real, NX, LN, KIND, true>(a, twn, tw2n, blockIdx.x);
 }
