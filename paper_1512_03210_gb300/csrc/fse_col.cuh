@@ -94,8 +94,8 @@ __device__ __forceinline__ void pass_prologue() {
 
 constexpr int kSMs = 152;  // GB300
 
-// Shape of a column pass along an axis of N points.
-template <typename Real, int N, int VAR>
+// Shape of a column pass along an axis of N points; THIN: of its narrower tiles.
+template <typename Real, int N, int VAR, bool THIN = false>
 struct ColShape {
   typedef typename LaneOf<Real>::T L;
   static constexpr int CW = sizeof(L) / sizeof(Real);  // columns per 16-byte element
@@ -112,9 +112,25 @@ struct ColShape {
   // 256^2 runs: 40.4 -> 37.4 and 40.7 -> 37.9 us per 50 runs). Length 96 takes
   // the eight-element plan everywhere (12 x 8 leaves a third of the threads
   // idle while the tile is loaded), and so do the shortest axes.
-  static constexpr int TT = (sizeof(Real) == 4 && M == 512 && VAR == COL_KHAT) ? 32 : 0;
-  static constexpr bool SLIM = VAR == COL_KIN2 || (VAR == COL_KHAT2 && M <= 256) || (!TWO && M == 96) || N <= 32;
-  typedef FftCfg<Real, M, TT, SLIM> F;
+  // Narrow tiles are a chain of latencies too: theirs is the plan of at most
+  // eight elements, with a thread for every item of radix 4 or more (2D passes
+  // keep their radices, so that a run's bits do not depend on how many advance
+  // together). Two steps: 16 x 16 x 128 39 -> 32 us, 12 x 64 x 24 58 -> 50, 256^2
+  // without interaction 38 -> 32, 192 x 96 55 -> 46.
+  static constexpr bool D2 = VAR == COL_KIN2 || VAR == COL_KHAT2;
+  static constexpr bool SLIM2 = VAR == COL_KIN2 || (VAR == COL_KHAT2 && M <= 256);
+  static constexpr bool SLIM = SLIM2 || (!TWO && M == 96) || N <= 32 || (THIN && !D2);
+  __host__ __device__ static constexpr int threads() {
+    if (sizeof(Real) == 8) return 0;
+    if (!THIN) return M == 512 && VAR == COL_KHAT ? 32 : 0;
+    if (D2 && !SLIM2) return 0;
+    const FftPlan p = fft_plan_slim(M);
+    int r = p.r[0];
+    for (int i = 1; i < p.np; ++i) r = p.r[i] < r ? p.r[i] : r;
+    const int t = M / (r < 4 ? 4 : r);
+    return t < p.T || t > 128 ? p.T : t;
+  }
+  typedef FftCfg<Real, M, threads(), SLIM> F;
   static constexpr int T = F::T;
   // Tile widths in elements: wide tiles move rows of 128 (64) bytes; the
   // narrow one is as few columns as still fill a warp, for grids whose wide
@@ -127,7 +143,7 @@ struct ColShape {
   }
   __host__ __device__ static constexpr int narrow() {
     int w = 1;
-    while (w * T < 32) w *= 2;
+    while (w * ColShape<Real, N, VAR, true>::T < 32) w *= 2;
     return w < wide() ? w : wide();
   }
   // between the two where they lie far apart
@@ -136,7 +152,8 @@ struct ColShape {
 
 template <typename Real, int N, int VAR, int NP>
 struct ColCfg {
-  typedef ColShape<Real, N, VAR> S;
+  static constexpr int WIDE = ColShape<Real, N, VAR>::wide();
+  typedef ColShape<Real, N, VAR, (NP < WIDE)> S;
   typedef typename S::F F;
   static constexpr int M = S::M, T = S::T, NT = NP * T, E = F::E;
   static constexpr int NC = S::CW * NP;  // columns per tile
@@ -309,7 +326,7 @@ __device__ __forceinline__ void col_tile(const ColArgs& a, const MulArgs& m, con
   // then a chain of memory latencies. The constant tables it will read (twiddles,
   // kinetic factors, C^) come into L1 or shared memory before the wait for the
   // previous pass, which they do not depend on.
-  constexpr bool EARLY = PDL && NP < K::S::wide();
+  constexpr bool EARLY = PDL && NP < K::WIDE;
   if constexpr (EARLY && F::P.np > 1) {
     unsigned x = F::template warm_table<VAR == COL_CROPI, K::S::EXACT, NT>(tw, tid);
     if constexpr (K::S::KIN || K::S::KHAT) x ^= F::template warm_table<true, K::S::EXACT, NT>(tw, tid);
