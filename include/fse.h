@@ -225,8 +225,9 @@ fse_status fse_plan_profile_read(fse_plan_t plan, double* ms, long long* count);
  * Many independent 2D runs (each the scheme of Section 4.2, Eqs. tssp1-tssp3,
  * with its own grid size, s, m, Omega, beta, lambda, dt and trap) advanced
  * together: runs of equal grid size share one launch per pass and one kernel
- * transform; a run advanced in a batch is bit-identical to the same run
- * advanced alone with fse_step. Requirements: dim 2, FSE_F32, renormalize 0, order 2, no lattice,
+ * transform; a run advanced in a batch has the bits of the same run advanced
+ * alone with fse_step, up to the rounding of the trap's coefficients to float
+ * (formed on the device from dt, not from the window's ends). Requirements: dim 2, FSE_F32, renormalize 0, order 2, no lattice,
  * one box, one kernel (none or Coulomb), one exponent mu and one Gaussian-sum
  * fit (gs_delta, gs_h, gs_tmin after defaults) for the whole batch. */
 typedef struct fse_batch* fse_batch_t;

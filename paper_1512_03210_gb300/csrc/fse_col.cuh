@@ -18,7 +18,7 @@
 
 namespace fse {
 
-enum { MUL_NONE = 0, MUL_KIN = 1, MUL_COULOMB = 2, MUL_DDI = 3 };
+enum { MUL_KIN = 1, MUL_COULOMB = 2, MUL_DDI = 3 };
 enum { COL_FWD = 0, COL_INV = 1, COL_PADF = 2, COL_CROPI = 3, COL_KIN = 4, COL_KHAT = 5, COL_KIN2 = 6, COL_KHAT2 = 7, COL_RMUL = 8, COL_DY = 9, COL_LZ = 10 };
 
 struct ColArgs {

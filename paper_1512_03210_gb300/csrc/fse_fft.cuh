@@ -13,21 +13,6 @@ template <> struct Cplx<double> { typedef double2 T; };
 __device__ __forceinline__ float2 mk(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ double2 mk(double a, double b) { return make_double2(a, b); }
 
-template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return mk(a.x + b.x, a.y + b.y); }
-template <typename C> __device__ __forceinline__ C csub(C a, C b) { return mk(a.x - b.x, a.y - b.y); }
-template <typename C> __device__ __forceinline__ C cmul(C a, C b) {
-  return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-// a * conj(b)
-template <typename C> __device__ __forceinline__ C cmulc(C a, C b) {
-  return mk(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
-}
-template <typename C> __device__ __forceinline__ C cconj(C a) { return mk(a.x, -a.y); }
-// multiply by -i (DIR < 0) or +i (DIR > 0)
-template <int DIR, typename C> __device__ __forceinline__ C mul_i(C a) {
-  return DIR < 0 ? mk(a.y, -a.x) : mk(-a.y, a.x);
-}
-
 // Asynchronous 4/8/16-byte global -> shared copy (cp.async, completes in the
 // background) and the wait for all of a thread's outstanding copies.
 template <int BYTES>
@@ -41,10 +26,6 @@ __device__ __forceinline__ void cp_async(void* smem, const void* gmem) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-// wait until at most N committed groups of this thread are still in flight
-template <int N> __device__ __forceinline__ void cp_async_wait_group() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
 // Bulk prefetch of a contiguous global range into L2 (address and size
 // multiples of 16 bytes); no completion to wait for.
 __device__ __forceinline__ void prefetch_l2_bulk(const void* gmem, unsigned bytes) {
@@ -60,38 +41,6 @@ __device__ __forceinline__ float norm_err(float c, float s) {
   const float pa = a * a, ea = fmaf(a, a, -pa);
   const float pb = b * b, eb = fmaf(b, b, -pb);
   return ((pa - 1.0f) + pb) + (ea + eb);
-}
-
-// Twiddle m of the table: rounded pair w and its remainder l (EXACT float path;
-// otherwise l = w unused). The transforms multiply with twiddle_apply,
-// conjugated for the inverse transform.
-template <bool EXACT, typename C>
-__device__ __forceinline__ void twiddle_load(const C* __restrict__ tw, int m, C& w, C& l) {
-  w = __ldg(&tw[2 * m]);
-  if constexpr (EXACT && sizeof(C) == 8) l = __ldg(&tw[2 * m + 1]);
-  else l = w;
-}
-template <int DIR, bool EXACT, typename C>
-__device__ __forceinline__ C twiddle_apply(C v, C w, C l) {
-  if constexpr (EXACT && sizeof(C) == 8) {
-    if constexpr (DIR < 0) {
-      const float lr = v.x * l.x - v.y * l.y, li = v.x * l.y + v.y * l.x;
-      return mk(fmaf(v.x, w.x, fmaf(-v.y, w.y, lr)), fmaf(v.x, w.y, fmaf(v.y, w.x, li)));
-    } else {
-      const float lr = v.x * l.x + v.y * l.y, li = v.y * l.x - v.x * l.y;
-      return mk(fmaf(v.x, w.x, fmaf(v.y, w.y, lr)), fmaf(-v.x, w.y, fmaf(v.y, w.x, li)));
-    }
-  } else {
-    return DIR < 0 ? cmul(v, w) : cmulc(v, w);
-  }
-}
-
-// v times twiddle m of the table (conjugated for the inverse transform).
-template <int DIR, bool EXACT, typename C>
-__device__ __forceinline__ C twiddle_mul(C v, const C* __restrict__ tw, int m) {
-  C w, l;
-  twiddle_load<EXACT>(tw, m, w, l);
-  return twiddle_apply<DIR, EXACT>(v, w, l);
 }
 
 // v times the float pair (c, s) of a unit-modulus factor, with the pair's

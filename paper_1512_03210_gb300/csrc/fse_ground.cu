@@ -373,7 +373,7 @@ struct Gs {
   long long N;
   int blocks, nlines, tiles, stride;
   GsGrid g;
-  C *phin, *r, *rh, *p, *v, *s, *t, *w;  // w: the operator's work field; phin doubles as d_y u inside a product
+  C *phin, *r, *rh, *p, *v, *s, *t, *w;  // w: the operator's work field
   C* dy;
   Real *W, *pk, *Phi;
   double *part, *out, *sc;
@@ -641,8 +641,8 @@ extern "C" fse_status fse_ground_state(fse_plan_t P, void* psi, void* workspace,
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P->gs_join, cudaEventDisableTiming);
     if (e != cudaSuccess) return cuda_fail(P, e, "ground state stream");
   }
-  // the solve runs on a stream of the plan's own (capturable, unlike the
-  // legacy default stream), after and before the caller's stream
+  // the solve runs on a stream of the plan's own (see fse_plan::gs_stream),
+  // after and before the caller's stream
   cudaStream_t user = P->stream;
   cudaError_t e = cudaEventRecord(P->gs_fork, user);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(P->gs_stream, P->gs_fork, 0);

@@ -199,8 +199,6 @@ template <typename F> __device__ __forceinline__ void RunScale<float2>::grow(flo
   inv = p.inv;
 }
 
-template <typename L> __device__ __forceinline__ Vec<L> vzero() { return {lbc<L>(0.0), lbc<L>(0.0)}; }
-
 // head and tail of a constant in the lane's precision (folded at compile time)
 __device__ __forceinline__ void head_tail(double k, float2& h, float2& t) {
   h = make_float2((float)k, (float)k);
