@@ -352,7 +352,8 @@ fse_status observables(fse_plan* P, const void* psi_in, double t, const double* 
   o.s = std::sin(P->p.omega * t);
   // In a turned frame the moments give a trap's energy up to rounding of that of
   // its stiff axis in all directions: for a cloud along the soft axis of frequencies
-  // 100 : 1 it was 6e-14 off, summed point by point 1e-16, as it is beyond 2 : 1.
+  // 100 : 1 it was 6e-14 off, summed point by point 1e-16, as it is beyond 2 : 1
+  // (observables of 128^3 float32 fields without interaction 130 -> 180 us).
   const double stiff = std::fmax(o.g2[0], o.g2[1]), soft = std::fmin(o.g2[0], o.g2[1]);
   o.by_points = o.s != 0.0 && !(stiff <= 4.0 * soft);
   o.lat_amp = P->p.lat_amp;
